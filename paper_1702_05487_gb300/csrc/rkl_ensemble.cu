@@ -41,8 +41,8 @@ struct rkl_ensemble {
     int64_t* d_cstart = nullptr;
     int* d_clen = nullptr;
     int* d_pchunk = nullptr;
-    double* d_partials = nullptr;
-    double* d_pstats = nullptr;          // [nprob][3]
+    float* d_partials = nullptr;          // {max, min} per statistics chunk
+    double* d_pstats = nullptr;          // [nprob][2]: max, min
     double* h_pstats = nullptr;          // pinned
 
     x2::EnsProb* d_probs = nullptr;
@@ -140,7 +140,7 @@ rkl_status ens_stats(rkl_ensemble* e, const float* T_all)
     cudaError_t c = launch_stats_segmented(T_all, e->d_cstart, e->d_clen, e->nchunk, e->d_pchunk, e->nprob,
                                            e->d_partials, e->d_pstats, e->stream);
     if (c != cudaSuccess) return efail(e, RKL_ERR_CUDA, std::string("stats: ") + cudaGetErrorString(c));
-    ENS_CK(e, cudaMemcpyAsync(e->h_pstats, e->d_pstats, sizeof(double) * 3 * e->nprob, cudaMemcpyDeviceToHost,
+    ENS_CK(e, cudaMemcpyAsync(e->h_pstats, e->d_pstats, sizeof(double) * 2 * e->nprob, cudaMemcpyDeviceToHost,
                               e->stream));
     ENS_CK(e, cudaMemcpyAsync(e->h_status, e->d_status, sizeof(unsigned), cudaMemcpyDeviceToHost, e->stream));
     ENS_CK(e, cudaMemsetAsync(e->d_status, 0, sizeof(unsigned), e->stream));
@@ -256,7 +256,7 @@ rkl_status ens_choose_s(rkl_ensemble* e, const double* dt, std::vector<int>& s)
 {
     s.assign(e->nprob, 0);
     for (int p = 0; p < e->nprob; ++p) {
-        const double mx = e->h_pstats[3 * p], mn = e->h_pstats[3 * p + 1];
+        const double mx = e->h_pstats[2 * p], mn = e->h_pstats[2 * p + 1];
         if (!std::isfinite(mx) || !std::isfinite(mn)) return efail(e, RKL_ERR_NONFINITE, "T holds NaN or Inf");
         if (e->phys[p].kappa_model == RKL_KAPPA_SPITZER && !(mn > 0.0))
             return efail(e, RKL_ERR_NONPOSITIVE_T, "T must be > 0 under Spitzer kappa");
@@ -356,9 +356,9 @@ rkl_status rkl_ensemble_create(int nprob, const rkl_grid* grids, const rkl_phys*
     if ((c = cudaMalloc(&e->d_cstart, sizeof(int64_t) * e->nchunk)) != cudaSuccess) return bail(c, "chunks");
     if ((c = cudaMalloc(&e->d_clen, sizeof(int) * e->nchunk)) != cudaSuccess) return bail(c, "chunks");
     if ((c = cudaMalloc(&e->d_pchunk, sizeof(int) * (nprob + 1))) != cudaSuccess) return bail(c, "chunks");
-    if ((c = cudaMalloc(&e->d_partials, sizeof(double) * 3 * e->nchunk)) != cudaSuccess) return bail(c, "partials");
-    if ((c = cudaMalloc(&e->d_pstats, sizeof(double) * 3 * nprob)) != cudaSuccess) return bail(c, "stats");
-    if ((c = cudaMallocHost(&e->h_pstats, sizeof(double) * 3 * nprob)) != cudaSuccess) return bail(c, "stats");
+    if ((c = cudaMalloc(&e->d_partials, sizeof(float) * 2 * e->nchunk)) != cudaSuccess) return bail(c, "partials");
+    if ((c = cudaMalloc(&e->d_pstats, sizeof(double) * 2 * nprob)) != cudaSuccess) return bail(c, "stats");
+    if ((c = cudaMallocHost(&e->h_pstats, sizeof(double) * 2 * nprob)) != cudaSuccess) return bail(c, "stats");
     if ((c = cudaMalloc(&e->d_probs, sizeof(x2::EnsProb) * nprob)) != cudaSuccess) return bail(c, "probs");
     if ((c = cudaMallocHost(&e->h_probs, sizeof(x2::EnsProb) * nprob)) != cudaSuccess) return bail(c, "probs");
     if ((c = cudaMalloc(&e->d_work, sizeof(int))) != cudaSuccess) return bail(c, "work");

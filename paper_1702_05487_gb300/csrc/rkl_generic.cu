@@ -3,6 +3,8 @@
 // the FP64 and low-dimensional configurations and every case the tiled FP32
 // kernel does not cover; each cell evaluates the fluxes on all of its faces
 // straight from global memory (L1/L2 absorb the neighbour re-reads).
+#include <algorithm>
+
 #include "rkl_launch.h"
 
 namespace rkl {
@@ -327,63 +329,85 @@ cudaError_t flux_dispatch_ndim(const LaunchCfg& c, const void* grid, const void*
 }
 
 // ---------------------------------------------------------------------------
-// FP64 statistics (max, min, sum) in a fixed reduction order.
+// Statistics (max, min, sum) of a grid array in a fixed reduction order.
+//
+// The FP64 units of this GPU retire two lanes per SM and clock, so a 64-bit
+// compare per lane and shuffle step costs more than reading the array: with
+// FP64 folds the pass over 256^3 FP32 cells took 37 us against 10 us of
+// memory time, and 860 thousand FP64 cells took 32 us.  The extrema are
+// therefore kept in the data's own type (FP32) or as order-preserving
+// integers (FP64), both exact, with a NaN flag beside them; only the sum
+// (energy), and only when asked for, is FP64 arithmetic.
 
 template <typename R>
-__device__ __forceinline__ void acc(double v, double& mx, double& mn, double& sm)
-{
-    // NaN propagates into max and min so that callers can detect it
-    mx = (v > mx || v != v) ? v : mx;
-    mn = (v < mn || v != v) ? v : mn;
-    sm += v;
-}
+struct Ext;
 
-// Max and min are exact in the data's own type; the sum (energy) is
-// accumulated in FP64 and only when asked for (FP64 arithmetic is scarce on
-// this GPU, and dt_expl needs only the extrema).  Each block leaves its
-// partial {max, min, sum}; the block that finishes last (ticket counter at
-// partials[3 * gridDim.x], reset by that block) folds all partials in a
-// fixed order, so the result does not depend on which block is last.
-__device__ __forceinline__ void fold_mm(double vmx, double vmn, double& mx, double& mn)
-{
-    mx = (vmx > mx || vmx != vmx) ? vmx : mx;
-    mn = (vmn < mn || vmn != vmn) ? vmn : mn;
-}
+template <>
+struct Ext<float> {
+    float mx = -INFINITY, mn = INFINITY;
+    int nan = 0;
+    __device__ __forceinline__ void add(float v)
+    {
+        mx = fmaxf(mx, v);
+        mn = fminf(mn, v);
+        nan |= v != v;
+    }
+    __device__ __forceinline__ float max_value() const { return nan ? NAN : mx; }
+    __device__ __forceinline__ float min_value() const { return nan ? NAN : mn; }
+};
 
-template <bool SUM>
-__device__ __forceinline__ void block_fold(double& mx, double& mn, double& sm)
+template <>
+struct Ext<double> {
+    // the total order of the doubles as signed integers
+    static __device__ __forceinline__ long long key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffll); }
+    long long mx = key((long long)0xfff0000000000000ull), mn = 0x7ff0000000000000ll;    // -inf, +inf
+    int nan = 0;
+    __device__ __forceinline__ void add(double v)
+    {
+        const long long b = __double_as_longlong(v), k = key(b);
+        mx = max(mx, k);
+        mn = min(mn, k);
+        nan |= (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+    }
+    __device__ __forceinline__ double max_value() const { return nan ? NAN : __longlong_as_double(key(mx)); }
+    __device__ __forceinline__ double min_value() const { return nan ? NAN : __longlong_as_double(key(mn)); }
+};
+
+// Folds the block's extrema and (SUM) sum into thread 0 (256 threads).
+template <typename R, bool SUM>
+__device__ __forceinline__ void block_fold(Ext<R>& e, double& sm)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        fold_mm(__shfl_xor_sync(0xffffffffu, mx, o), __shfl_xor_sync(0xffffffffu, mn, o), mx, mn);
+        e.mx = max(e.mx, __shfl_xor_sync(0xffffffffu, e.mx, o));
+        e.mn = min(e.mn, __shfl_xor_sync(0xffffffffu, e.mn, o));
         if (SUM) sm += __shfl_xor_sync(0xffffffffu, sm, o);
     }
-    __shared__ double s[3][8];
+    __shared__ decltype(Ext<R>::mx) smx[8], smn[8];
+    __shared__ double ss[8];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) { s[0][w] = mx; s[1][w] = mn; s[2][w] = sm; }
+    e.nan = __syncthreads_or(e.nan);
+    if (l == 0) { smx[w] = e.mx; smn[w] = e.mn; ss[w] = sm; }
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int q = 1; q < 8; ++q) {
-            fold_mm(s[0][q], s[1][q], mx, mn);
-            sm += s[2][q];
+            e.mx = max(e.mx, smx[q]);
+            e.mn = min(e.mn, smn[q]);
+            if (SUM) sm += ss[q];
         }
     }
 }
 
+// The extrema (and sum) of T[0 .. n) over one grid of blocks or one block:
+// thread t0 of `stride` threads.
 template <typename R, bool SUM>
-__global__ void __launch_bounds__(256) stats_kernel(const R* __restrict__ T, int64_t n, double* partials,
-                                                    double* out, unsigned* status)
+__device__ __forceinline__ void thread_stats(const R* __restrict__ T, int64_t n, int64_t t0, int64_t stride, Ext<R>& e,
+                                             double& sm)
 {
-    R mx = -INFINITY, mn = INFINITY;
-    double sm = 0.0;
     auto fold = [&](R v) {
-        mx = (v > mx || v != v) ? v : mx;
-        mn = (v < mn || v != v) ? v : mn;
+        e.add(v);
         if (SUM) sm += (double)v;
     };
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (sizeof(R) == 4 && (n & 3) == 0 && (reinterpret_cast<uintptr_t>(T) & 15) == 0) {
         const float4* T4 = reinterpret_cast<const float4*>(T);
         const int64_t n4 = n / 4;
@@ -403,31 +427,54 @@ __global__ void __launch_bounds__(256) stats_kernel(const R* __restrict__ T, int
             fold((R)v.x); fold((R)v.y); fold((R)v.z); fold((R)v.w);
         }
     } else {
-        for (int64_t c = t0; c < n; c += stride) fold(T[c]);
+        int64_t c = t0;
+        for (; c + 3 * stride < n; c += 4 * stride) {
+            R v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = T[c + u * stride];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) fold(v[u]);
+        }
+        for (; c < n; c += stride) fold(T[c]);
     }
-    double dmx = (double)mx, dmn = (double)mn;
-    block_fold<SUM>(dmx, dmn, sm);
+}
+
+// Each block leaves its partial {max, min, sum}; the block that finishes
+// last (ticket counter at partials[3 * kStatsBlocks], reset by that block)
+// folds all partials in a fixed order, so the result does not depend on
+// which block is last.
+template <typename R, bool SUM>
+__global__ void __launch_bounds__(256) stats_kernel(const R* __restrict__ T, int64_t n, double* partials,
+                                                    double* out, unsigned* status)
+{
+    Ext<R> e;
+    double sm = 0.0;
+    thread_stats<R, SUM>(T, n, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, e, sm);
+    block_fold<R, SUM>(e, sm);
     __shared__ bool last;
-    unsigned* ticket = reinterpret_cast<unsigned*>(partials + 3 * gridDim.x);
+    unsigned* ticket = reinterpret_cast<unsigned*>(partials + 3 * kStatsBlocks);
     if (threadIdx.x == 0) {
-        partials[3 * blockIdx.x + 0] = dmx;
-        partials[3 * blockIdx.x + 1] = dmn;
-        partials[3 * blockIdx.x + 2] = sm;
+        // the extrema in the data's own type, at the head of their slots
+        *reinterpret_cast<R*>(&partials[3 * blockIdx.x]) = e.max_value();
+        *reinterpret_cast<R*>(&partials[3 * blockIdx.x + 1]) = e.min_value();
+        if (SUM) partials[3 * blockIdx.x + 2] = sm;
         __threadfence();
         last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    dmx = -INFINITY; dmn = INFINITY; sm = 0.0;
+    e = Ext<R>();
+    sm = 0.0;
     for (int q = threadIdx.x; q < (int)gridDim.x; q += blockDim.x) {
-        fold_mm(__ldcg(&partials[3 * q]), __ldcg(&partials[3 * q + 1]), dmx, dmn);
-        sm += __ldcg(&partials[3 * q + 2]);
+        e.add(__ldcg(reinterpret_cast<const R*>(&partials[3 * q])));
+        e.add(__ldcg(reinterpret_cast<const R*>(&partials[3 * q + 1])));
+        if (SUM) sm += __ldcg(&partials[3 * q + 2]);
     }
-    block_fold<SUM>(dmx, dmn, sm);
+    block_fold<R, SUM>(e, sm);
     if (threadIdx.x == 0) {
-        out[0] = dmx;
-        out[1] = dmn;
+        out[0] = (double)e.max_value();
+        out[1] = (double)e.min_value();
         out[2] = sm;
         unsigned st = status ? *status : 0u;
         out[3] = (double)st;
@@ -468,7 +515,9 @@ cudaError_t launch_flux_generic(const LaunchCfg& c, const void* grid, const void
 cudaError_t launch_stats(int dtype, const void* T, int64_t n, double* partials, double* out,
                          unsigned* status, cudaStream_t st, bool need_sum)
 {
-    const int nb = kStatsBlocks;
+    // two 16-byte loads a thread at least: more blocks only queue at the ticket
+    const int per = dtype == 1 ? 1024 : 2048;
+    const int nb = (int)std::min<int64_t>(kStatsBlocks, (n + per - 1) / per);
     if (dtype == 1) {
         const double* Td = static_cast<const double*>(T);
         if (need_sum) stats_kernel<double, true><<<nb, 256, 0, st>>>(Td, n, partials, out, status);
@@ -482,79 +531,55 @@ cudaError_t launch_stats(int dtype, const void* T, int64_t n, double* partials, 
 }
 
 // ---------------------------------------------------------------------------
-// Segmented FP64 statistics of the problems of an ensemble: block c folds
-// chunk c (cells [cstart[c], cstart[c] + clen[c]) of one problem), then one
-// warp per problem folds that problem's chunks pchunk[p] .. pchunk[p+1]-1.
+// Segmented extrema of the problems of an ensemble: block c folds chunk c
+// (cells [cstart[c], cstart[c] + clen[c]) of one problem), then one warp per
+// problem folds that problem's chunks pchunk[p] .. pchunk[p+1]-1.  FP32 folds
+// (see Ext): 33.5 million cells took 236 us with FP64 ones.
 
 namespace {
 
 __global__ void __launch_bounds__(256) seg_stats_kernel(const float* __restrict__ T, const int64_t* cstart,
-                                                        const int* clen, double* partials)
+                                                        const int* clen, float2* partials)
 {
-    double mx = -INFINITY, mn = INFINITY, sm = 0.0;
-    const int64_t s0 = cstart[blockIdx.x];
-    const int len = clen[blockIdx.x];
-    for (int i = threadIdx.x; i < len; i += blockDim.x) acc<float>((double)T[s0 + i], mx, mn, sm);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        double omx = __shfl_xor_sync(0xffffffffu, mx, o);
-        double omn = __shfl_xor_sync(0xffffffffu, mn, o);
-        mx = (omx > mx || omx != omx) ? omx : mx;
-        mn = (omn < mn || omn != omn) ? omn : mn;
-        sm += __shfl_xor_sync(0xffffffffu, sm, o);
-    }
-    __shared__ double s[3][8];
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) { s[0][w] = mx; s[1][w] = mn; s[2][w] = sm; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int q = 1; q < 8; ++q) {
-            mx = (s[0][q] > mx || s[0][q] != s[0][q]) ? s[0][q] : mx;
-            mn = (s[1][q] < mn || s[1][q] != s[1][q]) ? s[1][q] : mn;
-            sm += s[2][q];
-        }
-        partials[3 * blockIdx.x + 0] = mx;
-        partials[3 * blockIdx.x + 1] = mn;
-        partials[3 * blockIdx.x + 2] = sm;
-    }
+    Ext<float> e;
+    double none = 0.0;
+    thread_stats<float, false>(T + cstart[blockIdx.x], clen[blockIdx.x], threadIdx.x, blockDim.x, e, none);
+    block_fold<float, false>(e, none);
+    if (threadIdx.x == 0) partials[blockIdx.x] = make_float2(e.max_value(), e.min_value());
 }
 
-__global__ void seg_stats_final_kernel(const double* partials, const int* pchunk, int nprob, double* out)
+__global__ void seg_stats_final_kernel(const float2* partials, const int* pchunk, int nprob, double* out)
 {
     const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int l = threadIdx.x & 31;
     if (p >= nprob) return;
-    double mx = -INFINITY, mn = INFINITY, sm = 0.0;
+    Ext<float> e;
     for (int q = pchunk[p] + l; q < pchunk[p + 1]; q += 32) {
-        double a = partials[3 * q], b = partials[3 * q + 1];
-        mx = (a > mx || a != a) ? a : mx;
-        mn = (b < mn || b != b) ? b : mn;
-        sm += partials[3 * q + 2];
+        e.add(partials[q].x);
+        e.add(partials[q].y);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        double omx = __shfl_xor_sync(0xffffffffu, mx, o);
-        double omn = __shfl_xor_sync(0xffffffffu, mn, o);
-        mx = (omx > mx || omx != omx) ? omx : mx;
-        mn = (omn < mn || omn != omn) ? omn : mn;
-        sm += __shfl_xor_sync(0xffffffffu, sm, o);
+        e.mx = fmaxf(e.mx, __shfl_xor_sync(0xffffffffu, e.mx, o));
+        e.mn = fminf(e.mn, __shfl_xor_sync(0xffffffffu, e.mn, o));
+        e.nan |= __shfl_xor_sync(0xffffffffu, e.nan, o);
     }
     if (l == 0) {
-        out[3 * p + 0] = mx;
-        out[3 * p + 1] = mn;
-        out[3 * p + 2] = sm;
+        out[2 * p + 0] = (double)e.max_value();
+        out[2 * p + 1] = (double)e.min_value();
     }
 }
 
 }  // namespace
 
 cudaError_t launch_stats_segmented(const float* T, const int64_t* cstart, const int* clen, int nchunk,
-                                   const int* pchunk, int nprob, double* partials, double* out, cudaStream_t st)
+                                   const int* pchunk, int nprob, float* partials, double* out, cudaStream_t st)
 {
-    seg_stats_kernel<<<nchunk, 256, 0, st>>>(T, cstart, clen, partials);
+    float2* part = reinterpret_cast<float2*>(partials);
+    seg_stats_kernel<<<nchunk, 256, 0, st>>>(T, cstart, clen, part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    seg_stats_final_kernel<<<(nprob + 7) / 8, 256, 0, st>>>(partials, pchunk, nprob, out);
+    seg_stats_final_kernel<<<(nprob + 7) / 8, 256, 0, st>>>(part, pchunk, nprob, out);
     return cudaGetLastError();
 }
 

@@ -92,7 +92,7 @@ bool pair_stage_supported(const LaunchCfg& c, const KGrid<float>& g);
 cudaError_t launch_stage_pair(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
                               void* Yj1, unsigned* status, int nzchunk, cudaStream_t st);
 
-// FP64 statistics of a grid array: max, min and sum (fixed-order, deterministic).
+// Statistics of a grid array: max, min (exact) and FP64 sum (fixed-order, deterministic).
 // partials must hold 3 * kStatsBlocks + 1 doubles, the last one zero before
 // the first call (a ticket counter the pass leaves at zero); out receives {max, min, sum}
 // followed by the status word (as a double), which is then cleared.
@@ -100,10 +100,11 @@ constexpr int kStatsBlocks = 1216;   // 8 x 152 SMs
 cudaError_t launch_stats(int dtype, const void* T, int64_t n, double* partials, double* out,
                          unsigned* status, cudaStream_t st, bool need_sum = true);
 
-// FP64 {max, min, sum} per problem of an ensemble (FP32 data), from a chunk
-// table: chunk c covers cells [cstart[c], cstart[c] + clen[c]); problem p
-// owns chunks pchunk[p] .. pchunk[p+1]-1.  out receives 3 doubles per problem.
+// {max, min} per problem of an ensemble (FP32 data), from a chunk table:
+// chunk c covers cells [cstart[c], cstart[c] + clen[c]); problem p owns chunks
+// pchunk[p] .. pchunk[p+1]-1.  partials holds 2 floats per chunk (8-byte
+// aligned); out receives 2 doubles per problem.
 cudaError_t launch_stats_segmented(const float* T, const int64_t* cstart, const int* clen, int nchunk,
-                                   const int* pchunk, int nprob, double* partials, double* out, cudaStream_t st);
+                                   const int* pchunk, int nprob, float* partials, double* out, cudaStream_t st);
 
 }  // namespace rkl
