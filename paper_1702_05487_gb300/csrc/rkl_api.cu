@@ -217,6 +217,9 @@ rkl_status check_plan(rkl_plan* p)
     return RKL_OK;
 }
 
+// 32-column tiles leave fewer columns idle than 64-column ones.
+bool narrow_tiles(int nx) { return (nx + 31) / 32 * 32 < (nx + 63) / 64 * 64; }
+
 // Launch one stage (or M) on stream st (the plan's stream, or the capture
 // stream while a graph is being recorded).
 rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, double mt, double gt,
@@ -228,9 +231,7 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
         bool al = aligned16(io.Y0) && aligned16(io.MY0) && aligned16(io.Yjm1) && aligned16(io.Yjm2) &&
                   aligned16(io.Yj) && aligned16(io.b);
         if ((p->variant == 0 || p->variant == 10 || p->variant == 11) && p->xqok && al) {
-            // automatic choice: 32-column tiles where they leave fewer columns idle
-            const int nx = (int)p->gf.n[0];
-            const bool narrow = p->variant == 11 || (p->variant == 0 && (nx + 31) / 32 * 32 < (nx + 63) / 64 * 64);
+            const bool narrow = p->variant == 11 || (p->variant == 0 && narrow_tiles(p->gf.n[0]));
             e = launch_stage_xq(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk, st, narrow ? 32 : 64);
         }
         else if (p->x2ok && al && (p->variant == 0 || (p->variant >= 3 && p->variant <= 9)))
@@ -899,8 +900,13 @@ rkl_status rkl_plan_autotune(rkl_plan* p, double dt, const void* T, const void* 
         for (int nz : {0, -1, 32}) cands.push_back({8, nz});
     if (p->xqok)
         for (int nz : {0, 16, 32}) {
-            cands.push_back({10, nz});
-            cands.push_back({11, nz});
+            // below 64 Ki cells a limited stage is bound by launch latency
+            // (3-4 us on either kernel): the search stays with the
+            // paired-cell build there
+            if (!lim || p->ncell >= 65536) cands.push_back({10, nz});
+            // 32-column tiles only where they leave fewer columns idle (the
+            // limited build has 64-column tiles only)
+            if (!lim && narrow_tiles(p->gf.n[0])) cands.push_back({11, nz});
         }
     void* scratch = nullptr;
     RKL_CK(p, cudaMalloc(&scratch, (size_t)p->ncell * p->esize));
