@@ -53,6 +53,7 @@ struct rkl_plan {
     void* ybuf4 = nullptr;             // fourth stage buffer of the two-stage kernel (allocated on use)
     bool pairok = false;               // two-stage kernel applies to the grid
     bool xqok = false;                 // row-pair kernel applies to the grid
+    bool colok = false;                // column-march kernel applies to the grid
     void* my0 = nullptr;
     double* d_partials = nullptr;
     // {max, min, sum, status} of the statistics pass, written by its last
@@ -238,13 +239,16 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
             e = launch_stage_x2(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk,
                                 p->variant == 4 ? 3 : (p->variant == 9 ? 6 : 2), st, p->variant == 6,
                                 p->variant == 7, p->variant == 8);
+        else if (p->colok && p->variant != 1 && p->variant != 2)
+            e = launch_stage_col(p->cfg, p->gf, p->pf, io, cf, p->d_status, st);
         else if (p->fast && al && (p->variant == 0 || p->variant == 2))
             e = launch_stage_fast(p->cfg, p->gf, p->pf, io, cf, p->d_status, st);
         else
             e = launch_stage_generic(p->cfg, &p->gf, &p->pf, io, &cf, p->d_status, st);
     } else {
         KCoef<double> cf{mu, nu, mt, gt};
-        e = launch_stage_generic(p->cfg, &p->gd, &p->pd, io, &cf, p->d_status, st);
+        if (p->colok && p->variant != 1) e = launch_stage_col(p->cfg, p->gd, p->pd, io, cf, p->d_status, st);
+        else e = launch_stage_generic(p->cfg, &p->gd, &p->pd, io, &cf, p->d_status, st);
     }
     if (e != cudaSuccess) return cuda_fail(p, e, "stage launch");
     return RKL_OK;
@@ -617,6 +621,10 @@ rkl_status rkl_plan_create(const rkl_grid* grid, const rkl_phys* phys, void* cud
     p->x2ok = g.dtype == RKL_F32 && x2_stage_supported(p->cfg, p->gf);
     p->pairok = g.dtype == RKL_F32 && pair_stage_supported(p->cfg, p->gf);
     p->xqok = g.dtype == RKL_F32 && xq_stage_supported(p->cfg, p->gf);
+    // a limiter floor inside the temperature range decides face by face on
+    // FP32 rounding, so FP32 plans with one keep the kernels they had
+    p->colok = col_stage_supported(g.dtype, g.ndim, p->gf.n, p->gf.plane) &&
+               (g.dtype == RKL_F64 || !p->cfg.limiter || p->cfg.lim_all);
 
     rkl_plan* P = p;
     auto bail = [&](cudaError_t e, const char* where) {
@@ -908,6 +916,8 @@ rkl_status rkl_plan_autotune(rkl_plan* p, double dt, const void* T, const void* 
             // limited build has 64-column tiles only)
             if (!lim && narrow_tiles(p->gf.n[0])) cands.push_back({11, nz});
         }
+    // kernels without a number of their own: the automatic choice
+    if (p->colok) cands.push_back({0, 0});
     void* scratch = nullptr;
     RKL_CK(p, cudaMalloc(&scratch, (size_t)p->ncell * p->esize));
     cudaEvent_t a = nullptr, e = nullptr;
