@@ -53,6 +53,7 @@ struct rkl_plan {
     void* ybuf4 = nullptr;             // fourth stage buffer of the two-stage kernel (allocated on use)
     bool pairok = false;               // two-stage kernel applies to the grid
     bool xqok = false;                 // row-pair kernel applies to the grid
+    bool xgok = false;                 // row-pair kernel for any width and boundary applies
     bool colok = false;                // column-march kernel applies to the grid
     void* my0 = nullptr;
     double* d_partials = nullptr;
@@ -235,6 +236,8 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
             const bool narrow = p->variant == 11 || (p->variant == 0 && narrow_tiles(p->gf.n[0]));
             e = launch_stage_xq(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk, st, narrow ? 32 : 64);
         }
+        else if (p->xgok && al && p->variant == 0)
+            e = launch_stage_xg(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk, st);
         else if (p->x2ok && al && (p->variant == 0 || (p->variant >= 3 && p->variant <= 9)))
             e = launch_stage_x2(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk,
                                 p->variant == 4 ? 3 : (p->variant == 9 ? 6 : 2), st, p->variant == 6,
@@ -621,6 +624,7 @@ rkl_status rkl_plan_create(const rkl_grid* grid, const rkl_phys* phys, void* cud
     p->x2ok = g.dtype == RKL_F32 && x2_stage_supported(p->cfg, p->gf);
     p->pairok = g.dtype == RKL_F32 && pair_stage_supported(p->cfg, p->gf);
     p->xqok = g.dtype == RKL_F32 && xq_stage_supported(p->cfg, p->gf);
+    p->xgok = g.dtype == RKL_F32 && xg_stage_supported(p->cfg, p->gf);
     // a limiter floor inside the temperature range decides face by face on
     // FP32 rounding, so FP32 plans with one keep the kernels they had
     p->colok = col_stage_supported(g.dtype, g.ndim, p->gf.n, p->gf.plane) &&
@@ -917,7 +921,7 @@ rkl_status rkl_plan_autotune(rkl_plan* p, double dt, const void* T, const void* 
             if (!lim && narrow_tiles(p->gf.n[0])) cands.push_back({11, nz});
         }
     // kernels without a number of their own: the automatic choice
-    if (p->colok) cands.push_back({0, 0});
+    if (p->colok || (p->xgok && !p->xqok)) cands.push_back({0, 0});
     void* scratch = nullptr;
     RKL_CK(p, cudaMalloc(&scratch, (size_t)p->ncell * p->esize));
     cudaEvent_t a = nullptr, e = nullptr;

@@ -92,6 +92,14 @@ cudaError_t launch_stage_xq(const LaunchCfg& c, const KGrid<float>& g, const KPh
                             const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st,
                             int txw = 64);
 
+// Row-pair FP32 3D stage kernel for any width and either boundary (rows
+// copied in 4-byte pieces, 64-column tiles): no limiter or the limiter at
+// every face, fewer than 2^31 cells, 16-byte aligned arrays; nzchunk <= 0
+// picks the chunk length.
+bool xg_stage_supported(const LaunchCfg& c, const KGrid<float>& g);
+cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
+                            const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st);
+
 // Two-stage paired-cell FP32 3D kernel: stages j (io, coefficients at
 // io.coef_tab[4 j]) and j + 1 (written to Yj1) in one pass, 60 x 7 tiles of
 // nzchunk planes.  Periodic grids with nx % 4 == 0 only.  Neither output may

@@ -161,6 +161,24 @@ cudaError_t launch_stage_xq(const LaunchCfg& c, const KGrid<float>& g, const KPh
     return xq::launch_q_mode<false, false, 64, false>(io.mode, g, p, a, coef, status, nzchunk, st);
 }
 
+bool xg_stage_supported(const LaunchCfg& c, const KGrid<float>& g)
+{
+    // 65535 tiles of 8 rows
+    return c.dtype == 0 && c.ndim == 3 && (!c.limiter || c.lim_all) && g.ncell < ((int64_t)1 << 31) &&
+           g.n[1] <= 8 * 65535;
+}
+
+cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
+                            const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st)
+{
+    if (!xg_stage_supported(c, g)) return cudaErrorNotSupported;
+    const x2::FastArgs a = x2_args(io);
+    int nzc = nzchunk > 0 ? nzchunk : xq::auto_nzchunk_q(g, 64, xq::SmemQ<64>::TY);
+    nzc = std::max(nzc, (g.n[2] + 65534) / 65535);      // the grid's z limit
+    if (c.limiter) return xq::launch_q_gen_lim(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st);
+    return xq::launch_q_gen(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st);
+}
+
 cudaError_t launch_ensemble_xq(bool spitzer, bool saturate, const x2::EnsProb* probs, const x2::EnsSeg* segs,
                                int nseg, int total, int* work, unsigned* done, unsigned* status, int* abort_flag,
                                long long spin_limit, int grid, cudaStream_t st)

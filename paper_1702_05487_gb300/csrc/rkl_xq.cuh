@@ -31,7 +31,16 @@
 // Every face flux, slope, divergence term and recurrence update is the
 // same operation on the same operands, in the same order, as in the
 // paired-cell kernel (rkl_x2_tile.cuh), so the two kernels write the same
-// bits.  Periodic grids with nx % 4 == 0 and fewer than 2^31 cells.
+// bits.  Grids with fewer than 2^31 cells: periodic with nx % 4 == 0, or
+// (GEN builds) any width and either boundary.  A GEN build copies rows in
+// 4-byte pieces, one cell per lane, because 16-byte chunks of a row start
+// aligned in global memory only if nx % 4 == 0: a warp's copy of 32 cells is
+// then one or two 128-byte lines, so the shared-memory and L1 traffic stay
+// those of the 16-byte copies and the price is issue slots (33 copies a
+// thread and plane instead of 9).  Each lane's wrapped or clamped column and
+// row offsets are fixed per tile; Dirichlet ghosts of T are stored, not
+// copied.  201 x 150 x 99 stage: 138 us (one-cell tiled kernel) ->
+// 38 us; Dirichlet 192 x 128 x 96, constant kappa: 29 (paired-cell) -> 23 us.
 #pragma once
 
 #include <algorithm>
@@ -161,7 +170,57 @@ __device__ __forceinline__ Pos y_pos(const KGrid<float>& g, int t, int i0, int j
     return Pos{(unsigned)(j0 + row) * (unsigned)g.n[0] + (unsigned)(i0 + cc), (unsigned)((row * TX + cc) * 4)};
 }
 
-template <bool SP, bool SAT, int MODE, int TXW, bool KP0 = false, bool LIM = false>
+__device__ __forceinline__ void cp4(unsigned d, const void* s)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(s));
+}
+__device__ __forceinline__ void st1(unsigned d, float v)
+{
+    asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(d), "f"(v));
+}
+
+// Copy offsets of a thread in a GEN build: its columns (one per 32 of the
+// tile's width), the rows w, w + 4, ... of the tile with its halo, and, for
+// the first 2 ROWS threads, one halo cell (columns -1 and TX of every row).
+// Element offsets in a plane, wrapped (periodic) or clamped (Dirichlet);
+// ghost: bit k column k, bit 8 + k row k, bit 31 the halo cell.
+template <class SM>
+struct GenPos {
+    static constexpr int NC = SM::TX / 32, NR = (SM::ROWS + NWARPS - 1) / NWARPS;
+    unsigned col[NC], row[NR];
+    unsigned hsrc, hdst;
+    unsigned ghost;
+};
+
+template <class SM>
+__device__ __forceinline__ GenPos<SM> gen_pos(const KGrid<float>& g, int tid, int i0, int j0)
+{
+    GenPos<SM> n;
+    n.ghost = 0u;
+    const int lane = tid & 31, w = tid >> 5, nx = g.n[0], ny = g.n[1];
+    auto at = [&](int i, int m, bool& out) -> unsigned {
+        out = g.bc == 1 && (i < 0 || i >= m);
+        return (unsigned)(g.bc == 1 ? clampi(i, m) : x2::pmod(i, m));
+    };
+    bool o, q;
+#pragma unroll
+    for (int k = 0; k < n.NC; ++k) {
+        n.col[k] = at(i0 + 32 * k + lane, nx, o);
+        n.ghost |= o ? 1u << k : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < n.NR; ++k) {
+        n.row[k] = at(j0 + w + NWARPS * k - 1, ny, o) * (unsigned)nx;
+        n.ghost |= o ? 256u << k : 0u;
+    }
+    const int hr = tid >> 1, hc = (tid & 1) ? SM::TX : -1;
+    n.hsrc = at(j0 + hr - 1, ny, o) * (unsigned)nx + at(i0 + hc, nx, q);
+    n.hdst = tid < 2 * SM::ROWS ? (unsigned)(SM::off(hr - 1, hc) * 4) : ~0u;
+    n.ghost |= o || q ? 1u << 31 : 0u;
+    return n;
+}
+
+template <bool SP, bool SAT, int MODE, int TXW, bool KP0 = false, bool LIM = false, bool GEN = false>
 __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, const KPhys<float>& p,
                                        const x2::FastArgs& a, KCoef<float> cf, unsigned* status, int i0, int j0,
                                        int z0, int nzc)
@@ -183,8 +242,15 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
         cf.mu = t[0]; cf.nu = t[1]; cf.mt = t[2]; cf.gt = t[3];
     }
 
-    const Pos p0 = tb_pos<Smem>(g, tid, i0, j0), p1 = tb_pos<Smem>(g, tid + NTHREADS, i0, j0);
-    const Pos py = MODE == 2 ? y_pos<Smem>(g, tid, i0, j0) : Pos{0u, ~0u};
+    Pos p0{0u, ~0u}, p1{0u, ~0u}, py{0u, ~0u};
+    GenPos<Smem> gp;
+    if (GEN) {
+        gp = gen_pos<Smem>(g, tid, i0, j0);
+    } else {
+        p0 = tb_pos<Smem>(g, tid, i0, j0);
+        p1 = tb_pos<Smem>(g, tid + NTHREADS, i0, j0);
+        if (MODE == 2) py = y_pos<Smem>(g, tid, i0, j0);
+    }
     const float* bxp = a.b;
     const float* byp = a.b + g.ncell;
     const float* bzp = a.b + 2 * g.ncell;
@@ -198,12 +264,50 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
 
     // T and b of plane k, and (stages j >= 2) the Y bundle of plane k - 1
     auto load = [&](int k) {
-        int kz = z0 + k;                        // periodic: wrap the plane index
-        kz += kz < 0 ? nz : 0;
+        int kz = z0 + k;
+        const bool zg = GEN && g.bc == 1 && (kz < 0 || kz >= nz);
+        if (zg) kz = kz < 0 ? 0 : nz - 1;       // Dirichlet: ghosts, b of the nearest plane
+        kz += kz < 0 ? nz : 0;                  // periodic: wrap the plane index
         kz -= kz >= nz ? nz : 0;
         const unsigned pt = (unsigned)kz * plane;
         const unsigned ts = tbase + (unsigned)(tslot(k) * PLANE * 4);
         const unsigned bs = bbase + (unsigned)(bslot(k) * 3 * PLANE * 4);
+        if constexpr (GEN) {
+            auto copy = [&](unsigned x, unsigned d, bool ghost) {
+                if (ghost) st1(ts + d, g.bcv);
+                else cp4(ts + d, a.Tin + x);
+                cp4(bs + d, bxp + x);
+                cp4(bs + PLANE * 4 + d, byp + x);
+                cp4(bs + 2 * PLANE * 4 + d, bzp + x);
+            };
+#pragma unroll
+            for (int r = 0; r < gp.NR; ++r) {
+                if (w + NWARPS * r >= Smem::ROWS) break;
+                const unsigned d = (unsigned)(((w + NWARPS * r) * TX + lane) * 4);
+#pragma unroll
+                for (int m = 0; m < gp.NC; ++m)
+                    copy(gp.row[r] + gp.col[m] + pt, d + 128u * m, zg || (gp.ghost & ((256u << r) | (1u << m))));
+            }
+            if (gp.hdst != ~0u) copy(gp.hsrc + pt, gp.hdst, zg || (gp.ghost >> 31));
+            if (MODE == 2 && k >= 1) {
+                // plane k - 1 lies inside the chunk, so inside the grid
+                const unsigned ys = ybase + (unsigned)(yslot(k - 1) * 3 * TY * TX * 4);
+#pragma unroll
+                for (int r = 0; r < TY; r += NWARPS) {
+                    const unsigned x = (unsigned)(z0 + k - 1) * plane + (unsigned)(j0 + w + r) * (unsigned)nx +
+                                       (unsigned)(i0 + lane);
+                    const unsigned d = (unsigned)(((w + r) * TX + lane) * 4);
+#pragma unroll
+                    for (int m = 0; m < gp.NC; ++m)
+                        if (j0 + w + r < ny && i0 + lane + 32 * m < nx) {
+                            cp4(ys + d + 128u * m, a.Y0 + x + 32 * m);
+                            cp4(ys + TY * TX * 4 + d + 128u * m, a.Yjm2 + x + 32 * m);
+                            cp4(ys + 2 * TY * TX * 4 + d + 128u * m, a.MY0in + x + 32 * m);
+                        }
+                }
+            }
+            return;
+        }
         {
             const unsigned x = p0.src + pt;
             cp16(ts + p0.dst, a.Tin + x);
@@ -260,7 +364,18 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     float2 Tm0 = A.T0, Tm1 = A.T1, TmU = A.TU;
     float Tmr0 = A.r0, Tmr1 = A.r1;
 
-    const bool inx = i0 + c < nx;               // nx % 4 == 0: both cells or none
+    const bool inx = i0 + c < nx;               // both cells or none, unless GEN: then perhaps the first alone
+    const bool in2 = !GEN || i0 + c + 1 < nx;
+    const bool vec = !GEN || (nx & 1) == 0;     // pairs are 8-byte aligned
+    auto put = [&](float* o, float2 v) {
+        if (vec) *reinterpret_cast<float2*>(o) = v;
+        else {
+            o[0] = v.x;
+            if (in2) o[1] = v.y;
+        }
+    };
+    // the check's operand: an odd width's last pair repeats its first cell
+    auto seen = [&](float2 y) { return in2 ? y : bc2(y.x); };
     const bool in0 = inx && j0 + ra < ny, in1 = inx && j0 + rb < ny;
     int64_t cbase = ((int64_t)z0 * ny + (j0 + ra)) * nx + (i0 + c);
 
@@ -274,22 +389,23 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     float mnacc = INFINITY;
 
     auto emit = [&](int64_t o, float2 M, float2 To, float2 py0, float2 pyjm2, float2 pmy0) {
-        float2* out = reinterpret_cast<float2*>(a.out + o);
         if (MODE == 0) {
-            *out = M;
+            put(a.out + o, M);
         } else if (MODE == 1) {
-            if (a.MY0out) *reinterpret_cast<float2*>(a.MY0out + o) = M;
+            if (a.MY0out) put(a.MY0out + o, M);
             const float2 y = fma2(bc2(cf.mt), M, To);
-            nfacc = add2(nfacc, sub2(y, y));
-            if (SP) mnacc = fminf(mnacc, fminf(y.x, y.y));
-            *out = y;
+            put(a.out + o, y);
+            const float2 v = seen(y);
+            nfacc = add2(nfacc, sub2(v, v));
+            if (SP) mnacc = fminf(mnacc, fminf(v.x, v.y));
         } else {
             const float2 inc = fma2(bc2(cf.mu), sub2(To, py0),
                                     fma2(bc2(cf.nu), sub2(pyjm2, py0), fma2(bc2(cf.mt), M, mul2(bc2(cf.gt), pmy0))));
             const float2 y = add2(py0, inc);
-            nfacc = add2(nfacc, sub2(y, y));
-            if (SP) mnacc = fminf(mnacc, fminf(y.x, y.y));
-            *out = y;
+            put(a.out + o, y);
+            const float2 v = seen(y);
+            nfacc = add2(nfacc, sub2(v, v));
+            if (SP) mnacc = fminf(mnacc, fminf(v.x, v.y));
         }
     };
     // Tm0 / Tm1 hold T of plane qp when finish(qp) runs
@@ -429,18 +545,18 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     __syncthreads();
 }
 
-template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM>
+template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM, bool GEN>
 __global__ void __launch_bounds__(NTHREADS, kCtasPerSm)
 stage_q_kernel(KGrid<float> g, KPhys<float> p, x2::FastArgs a, KCoef<float> cf, unsigned* status, int nzchunk)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     SmemQ<TXW>& sm = *reinterpret_cast<SmemQ<TXW>*>(smem_raw);
     const int z0 = blockIdx.z * nzchunk;
-    tile_q<SP, SAT, MODE, TXW, KP0, LIM>(sm, g, p, a, cf, status, blockIdx.x * SmemQ<TXW>::TX, blockIdx.y * SmemQ<TXW>::TY,
+    tile_q<SP, SAT, MODE, TXW, KP0, LIM, GEN>(sm, g, p, a, cf, status, blockIdx.x * SmemQ<TXW>::TX, blockIdx.y * SmemQ<TXW>::TY,
                                z0, min(nzchunk, g.n[2] - z0));
 }
 
-template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM>
+template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM, bool GEN>
 cudaError_t launch_q(const KGrid<float>& g, const KPhys<float>& p, const x2::FastArgs& a, const KCoef<float>& cf,
                      unsigned* status, int nzchunk, cudaStream_t st)
 {
@@ -448,23 +564,23 @@ cudaError_t launch_q(const KGrid<float>& g, const KPhys<float>& p, const x2::Fas
     const int smem = (int)sizeof(SM);
     static bool attr_set = false;       // the attribute is per function, set once
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM>,
+        cudaError_t e = cudaFuncSetAttribute(stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM, GEN>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     const dim3 grid((g.n[0] + SM::TX - 1) / SM::TX, (g.n[1] + SM::TY - 1) / SM::TY, (g.n[2] + nzchunk - 1) / nzchunk);
-    stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM><<<grid, NTHREADS, smem, st>>>(g, p, a, cf, status, nzchunk);
+    stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM, GEN><<<grid, NTHREADS, smem, st>>>(g, p, a, cf, status, nzchunk);
     return cudaGetLastError();
 }
 
-template <bool SP, bool SAT, int TXW, bool KP0, bool LIM = false>
+template <bool SP, bool SAT, int TXW, bool KP0, bool LIM = false, bool GEN = false>
 cudaError_t launch_q_mode(int mode, const KGrid<float>& g, const KPhys<float>& p, const x2::FastArgs& a,
                           const KCoef<float>& cf, unsigned* status, int nzchunk, cudaStream_t st)
 {
-    if (mode == 0) return launch_q<SP, SAT, 0, TXW, KP0, LIM>(g, p, a, cf, status, nzchunk, st);
-    if (mode == 1) return launch_q<SP, SAT, 1, TXW, KP0, LIM>(g, p, a, cf, status, nzchunk, st);
-    return launch_q<SP, SAT, 2, TXW, KP0, LIM>(g, p, a, cf, status, nzchunk, st);
+    if (mode == 0) return launch_q<SP, SAT, 0, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st);
+    if (mode == 1) return launch_q<SP, SAT, 1, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st);
+    return launch_q<SP, SAT, 2, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st);
 }
 
 // Launches of the builds compiled in rkl_xq_sat.cu (saturated flux; kp0:
@@ -476,6 +592,14 @@ cudaError_t launch_q_sat(bool sp, bool kp0, int txw, int mode, const KGrid<float
 cudaError_t launch_q_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
                          cudaStream_t st);
+// GEN builds (rkl_xg.cu: classical and saturated flux, rkl_xg_lim.cu: MC
+// limiter; 64-column tiles).
+cudaError_t launch_q_gen(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
+                         const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
+                         cudaStream_t st);
+cudaError_t launch_q_gen_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
+                             const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
+                             cudaStream_t st);
 
 }  // namespace xq
 }  // namespace rkl
