@@ -325,6 +325,7 @@ col3_kernel(KGrid<R> g, KPhys<R> p, Args<R> a, KCoef<R> cf, unsigned* status, in
                                    L.b[1] + H.b[1], fk, p);
     };
 
+    chain_wait();
     Q A = read(-1), B = read(0);
     R Fzl = w < NW ? zface(A, B) : R(0);
     R Tmc = A.c, Tmr = A.r, Tmu = A.u;
@@ -386,6 +387,7 @@ col3_kernel(KGrid<R> g, KPhys<R> p, Args<R> a, KCoef<R> cf, unsigned* status, in
         Tmu = B.u;
         B = N;
     }
+    chain_release();
     if (bad) atomicOr(status, bad);
 }
 
@@ -447,6 +449,7 @@ col2_kernel(KGrid<R> g, KPhys<R> p, Args<R> a, KCoef<R> cf, unsigned* status, in
                                    L.b[1] + H.b[1], L.b[0] + H.b[0], R(0), fk, p);
     };
 
+    chain_wait();
     Q A = read(-1), B = read(0), N = read(1);
     R Fyl = yface(A, B);
     R Tmc = A.c, Tmr = A.r;
@@ -475,6 +478,7 @@ col2_kernel(KGrid<R> g, KPhys<R> p, Args<R> a, KCoef<R> cf, unsigned* status, in
         B = N;
         N = P;
     }
+    chain_release();
     if (bad) atomicOr(status, bad);
 }
 
@@ -517,7 +521,7 @@ inline int chunk3(int64_t cols, int nz)
 
 template <typename R, bool SP, bool SAT, bool LIM, bool CUBE>
 cudaError_t launch_nd(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, const Args<R>& a, const KCoef<R>& cf,
-                      unsigned* status, cudaStream_t st)
+                      unsigned* status, cudaStream_t st, bool chained)
 {
     if constexpr (sizeof(R) == 8) {
         if (c.ndim == 3) {
@@ -525,8 +529,8 @@ cudaError_t launch_nd(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, 
             const int bx = (g.n[0] + lpr - 1) / lpr, by = (g.n[1] + rows - 1) / rows;
             const int nzc = chunk3((int64_t)bx * by, g.n[2]);
             const dim3 grid(bx, by, (g.n[2] + nzc - 1) / nzc);
-            col3_kernel<R, SP, SAT, LIM, CUBE><<<grid, NT, 0, st>>>(g, p, a, cf, status, nzc, lpr);
-            return cudaGetLastError();
+            return launch_chained(col3_kernel<R, SP, SAT, LIM, CUBE>, grid, NT, 0, st, chained, g, p, a, cf, status, nzc,
+                                  lpr);
         }
     }
     const int ntx = (g.n[0] + 30) / 31;
@@ -534,22 +538,21 @@ cudaError_t launch_nd(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, 
     const int64_t warps = (int64_t)32 * sms();
     const int ch = (int)std::min<int64_t>(32, std::max<int64_t>(1, ((int64_t)ntx * g.n[1] + warps - 1) / warps));
     const int64_t items = (int64_t)ntx * ((g.n[1] + ch - 1) / ch);
-    col2_kernel<R, SP, SAT, LIM, CUBE><<<(unsigned)((items + NW2 - 1) / NW2), 32 * NW2, 0, st>>>(g, p, a, cf, status, ch,
-                                                                                            ntx, (int)items);
-    return cudaGetLastError();
+    return launch_chained(col2_kernel<R, SP, SAT, LIM, CUBE>, (unsigned)((items + NW2 - 1) / NW2), 32 * NW2, 0, st,
+                          chained, g, p, a, cf, status, ch, ntx, (int)items);
 }
 
 template <typename R, bool SP, bool SAT>
 cudaError_t launch_form(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, const Args<R>& a, const KCoef<R>& cf,
-                        unsigned* status, cudaStream_t st)
+                        unsigned* status, cudaStream_t st, bool chained)
 {
     bool cube = true;
     for (int d = 1; d < c.ndim; ++d) cube = cube && g.inv_dx[d] == g.inv_dx[0];
     if (c.limiter)
-        return cube ? launch_nd<R, SP, SAT, true, true>(c, g, p, a, cf, status, st)
-                    : launch_nd<R, SP, SAT, true, false>(c, g, p, a, cf, status, st);
-    return cube ? launch_nd<R, SP, SAT, false, true>(c, g, p, a, cf, status, st)
-                : launch_nd<R, SP, SAT, false, false>(c, g, p, a, cf, status, st);
+        return cube ? launch_nd<R, SP, SAT, true, true>(c, g, p, a, cf, status, st, chained)
+                    : launch_nd<R, SP, SAT, true, false>(c, g, p, a, cf, status, st, chained);
+    return cube ? launch_nd<R, SP, SAT, false, true>(c, g, p, a, cf, status, st, chained)
+                : launch_nd<R, SP, SAT, false, false>(c, g, p, a, cf, status, st, chained);
 }
 
 template <typename R>
@@ -561,10 +564,10 @@ cudaError_t launch(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, con
                     io.mode == 1 ? static_cast<R*>(io.MY0) : nullptr, static_cast<R*>(io.Yj),
                     static_cast<const R*>(io.coef_tab), io.j, io.mode};
     if (c.spitzer)
-        return c.saturate ? launch_form<R, true, true>(c, g, p, a, cf, status, st)
-                          : launch_form<R, true, false>(c, g, p, a, cf, status, st);
-    return c.saturate ? launch_form<R, false, true>(c, g, p, a, cf, status, st)
-                      : launch_form<R, false, false>(c, g, p, a, cf, status, st);
+        return c.saturate ? launch_form<R, true, true>(c, g, p, a, cf, status, st, io.chained)
+                          : launch_form<R, true, false>(c, g, p, a, cf, status, st, io.chained);
+    return c.saturate ? launch_form<R, false, true>(c, g, p, a, cf, status, st, io.chained)
+                      : launch_form<R, false, false>(c, g, p, a, cf, status, st, io.chained);
 }
 
 }  // namespace col

@@ -135,6 +135,14 @@ __device__ __forceinline__ int clampi(int i, int n)
     return i < 0 ? 0 : (i >= n ? n - 1 : i);
 }
 
+// Programmatic dependent launch (no effect in a launch without it):
+// chain_release lets the next kernel of the chain start its blocks as this
+// one's slots free up; chain_wait returns once the previous kernel has
+// finished and its writes are visible.  Nothing a stage writes may be touched
+// before chain_wait.
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 // Record a bad stage value in the device status word.
 template <typename R, bool SPITZER>
 __device__ __forceinline__ void check_value(R y, unsigned* status)

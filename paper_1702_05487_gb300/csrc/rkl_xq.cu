@@ -150,15 +150,15 @@ cudaError_t launch_stage_xq(const LaunchCfg& c, const KGrid<float>& g, const KPh
     // the limited build comes with 64-column tiles only
     if (c.limiter) txw = 64;
     if (nzchunk <= 0) nzchunk = xq::auto_nzchunk_q(g, txw, txw == 64 ? xq::SmemQ<64>::TY : xq::SmemQ<32>::TY);
-    if (c.limiter) return xq::launch_q_lim(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzchunk, st);
+    if (c.limiter) return xq::launch_q_lim(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzchunk, st, io.chained);
     if (c.saturate)
-        return xq::launch_q_sat(c.spitzer != 0, p.kperp == 0.f, txw, io.mode, g, p, a, coef, status, nzchunk, st);
+        return xq::launch_q_sat(c.spitzer != 0, p.kperp == 0.f, txw, io.mode, g, p, a, coef, status, nzchunk, st, io.chained);
     if (c.spitzer) {
-        if (txw == 32) return xq::launch_q_mode<true, false, 32, false>(io.mode, g, p, a, coef, status, nzchunk, st);
-        return xq::launch_q_mode<true, false, 64, false>(io.mode, g, p, a, coef, status, nzchunk, st);
+        if (txw == 32) return xq::launch_q_mode<true, false, 32, false>(io.mode, g, p, a, coef, status, nzchunk, st, io.chained);
+        return xq::launch_q_mode<true, false, 64, false>(io.mode, g, p, a, coef, status, nzchunk, st, io.chained);
     }
-    if (txw == 32) return xq::launch_q_mode<false, false, 32, false>(io.mode, g, p, a, coef, status, nzchunk, st);
-    return xq::launch_q_mode<false, false, 64, false>(io.mode, g, p, a, coef, status, nzchunk, st);
+    if (txw == 32) return xq::launch_q_mode<false, false, 32, false>(io.mode, g, p, a, coef, status, nzchunk, st, io.chained);
+    return xq::launch_q_mode<false, false, 64, false>(io.mode, g, p, a, coef, status, nzchunk, st, io.chained);
 }
 
 bool xg_stage_supported(const LaunchCfg& c, const KGrid<float>& g)
@@ -175,8 +175,8 @@ cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPh
     const x2::FastArgs a = x2_args(io);
     int nzc = nzchunk > 0 ? nzchunk : xq::auto_nzchunk_q(g, 64, xq::SmemQ<64>::TY);
     nzc = std::max(nzc, (g.n[2] + 65534) / 65535);      // the grid's z limit
-    if (c.limiter) return xq::launch_q_gen_lim(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st);
-    return xq::launch_q_gen(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st);
+    if (c.limiter) return xq::launch_q_gen_lim(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st, io.chained);
+    return xq::launch_q_gen(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st, io.chained);
 }
 
 cudaError_t launch_ensemble_xq(bool spitzer, bool saturate, const x2::EnsProb* probs, const x2::EnsSeg* segs,

@@ -332,6 +332,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
         }
     };
 
+    chain_wait();
     // groups: plane -1, then planes 0 .. PD; plane k's group also carries
     // the Y bundle of plane k - 1
     load(-1);
@@ -535,6 +536,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     }
     if (q < nzc) step(q, B, A);
     cp_wait<0>();
+    chain_release();
     __syncthreads();
     finish(nzc - 1);
     if (MODE != 0) {
@@ -558,7 +560,7 @@ stage_q_kernel(KGrid<float> g, KPhys<float> p, x2::FastArgs a, KCoef<float> cf, 
 
 template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM, bool GEN>
 cudaError_t launch_q(const KGrid<float>& g, const KPhys<float>& p, const x2::FastArgs& a, const KCoef<float>& cf,
-                     unsigned* status, int nzchunk, cudaStream_t st)
+                     unsigned* status, int nzchunk, cudaStream_t st, bool chained)
 {
     using SM = SmemQ<TXW>;
     const int smem = (int)sizeof(SM);
@@ -570,17 +572,17 @@ cudaError_t launch_q(const KGrid<float>& g, const KPhys<float>& p, const x2::Fas
         attr_set = true;
     }
     const dim3 grid((g.n[0] + SM::TX - 1) / SM::TX, (g.n[1] + SM::TY - 1) / SM::TY, (g.n[2] + nzchunk - 1) / nzchunk);
-    stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM, GEN><<<grid, NTHREADS, smem, st>>>(g, p, a, cf, status, nzchunk);
-    return cudaGetLastError();
+    return launch_chained(stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM, GEN>, grid, NTHREADS, smem, st, chained, g, p, a,
+                          cf, status, nzchunk);
 }
 
 template <bool SP, bool SAT, int TXW, bool KP0, bool LIM = false, bool GEN = false>
 cudaError_t launch_q_mode(int mode, const KGrid<float>& g, const KPhys<float>& p, const x2::FastArgs& a,
-                          const KCoef<float>& cf, unsigned* status, int nzchunk, cudaStream_t st)
+                          const KCoef<float>& cf, unsigned* status, int nzchunk, cudaStream_t st, bool chained)
 {
-    if (mode == 0) return launch_q<SP, SAT, 0, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st);
-    if (mode == 1) return launch_q<SP, SAT, 1, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st);
-    return launch_q<SP, SAT, 2, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st);
+    if (mode == 0) return launch_q<SP, SAT, 0, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st, chained);
+    if (mode == 1) return launch_q<SP, SAT, 1, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st, chained);
+    return launch_q<SP, SAT, 2, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st, chained);
 }
 
 // Launches of the builds compiled in rkl_xq_sat.cu (saturated flux; kp0:
@@ -588,18 +590,18 @@ cudaError_t launch_q_mode(int mode, const KGrid<float>& g, const KPhys<float>& p
 // 64-column tiles).
 cudaError_t launch_q_sat(bool sp, bool kp0, int txw, int mode, const KGrid<float>& g, const KPhys<float>& p,
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
-                         cudaStream_t st);
+                         cudaStream_t st, bool chained);
 cudaError_t launch_q_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
-                         cudaStream_t st);
+                         cudaStream_t st, bool chained);
 // GEN builds (rkl_xg.cu: classical and saturated flux, rkl_xg_lim.cu: MC
 // limiter; 64-column tiles).
 cudaError_t launch_q_gen(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
-                         cudaStream_t st);
+                         cudaStream_t st, bool chained);
 cudaError_t launch_q_gen_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                              const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
-                             cudaStream_t st);
+                             cudaStream_t st, bool chained);
 
 }  // namespace xq
 }  // namespace rkl
