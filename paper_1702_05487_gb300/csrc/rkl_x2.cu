@@ -99,7 +99,7 @@ bool x2_tmaps_supported(const LaunchCfg& c, const KGrid<float>& g)
 // give at least 3.5 waves of CTAs where the grid has that many.  Measured
 // on the 256^3 grid at five CTAs per SM: chunks of 20-24 planes (3.7-4.4
 // waves) 113 us per stage, 28-37 planes (2.4-3.4 waves) 116 us.  Grids with
-// fewer CTAs take chunks of 1 .. 48 planes: a chunk costs its planes and 2.5
+// less than one wave at 16 planes take chunks of 1 .. 48 planes: a chunk costs its planes and 2.5
 // for its prologue, a plane one latency-bound step until four CTAs share an
 // SM and the SM's throughput beyond (fitted to a sweep over 32^3 .. 128^3,
 // Dirichlet 192 x 128 x 96 and others, within 6% of the best length on
@@ -109,15 +109,16 @@ static int auto_nzchunk(const KGrid<float>& g, int occupancy)
 {
     const int64_t cols = (int64_t)((g.n[0] + x2::TX - 1) / x2::TX) * ((g.n[1] + x2::TY - 1) / x2::TY);
     const int64_t slots = (int64_t)ctas_per_sm(occupancy) * sm_count();
-    const bool many = cols * ((g.n[2] + 15) / 16) * 2 >= 7 * slots;
+    const int64_t at16 = cols * ((g.n[2] + 15) / 16);
+    const bool many = at16 * 2 >= 7 * slots, wave = at16 >= slots;
     int best = 32;
     double cost = 1e300;
-    for (int nzc = many ? 16 : 1; nzc <= 48; ++nzc) {
+    for (int nzc = wave ? 16 : 1; nzc <= 48; ++nzc) {
         const int64_t chunks = (g.n[2] + nzc - 1) / nzc;
         if (many && cols * chunks * 2 < 7 * slots) continue;
         const int64_t rounds = (cols * chunks + slots - 1) / slots;
         const double c = (std::min(nzc, g.n[2]) + 2.5) *
-                         (many ? (double)rounds : std::max(4.0, (double)(cols * chunks) / sm_count()));
+                         (wave ? (double)rounds : std::max(4.0, (double)(cols * chunks) / sm_count()));
         if (c < cost - 1e-9) {
             cost = c;
             best = nzc;

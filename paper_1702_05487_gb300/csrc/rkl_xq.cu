@@ -97,27 +97,29 @@ cudaError_t ensemble_launch_q(const x2::EnsProb* probs, const x2::EnsSeg* segs, 
 // Planes per CTA.  Grids with at least 3.5 waves of CTAs at 16 planes: among
 // 16 .. 64, the length that minimises (rounds of resident CTAs) x (planes +
 // halo cost), keeping the 3.5 waves (the paired-cell kernel's rule with this
-// kernel's tile and occupancy).  Smaller grids fill the chip with shorter
+// kernel's tile and occupancy); down to one wave at 16 planes the same cost
+// without that floor.  Grids below one wave fill the chip with shorter
 // chunks: with k CTAs per SM (mean), a chunk costs its planes and 1.5 for its
 // prologue, and a plane costs one latency-bound step (2.2 units) until about
 // two CTAs share an SM, then the SM's throughput, between the mean k and the
 // fullest SM's ceil(k).  Constants fitted to a sweep of 1 .. 64 planes over
-// 32^3 .. 192^3 and two uneven boxes; the choice is within 4% of the best
+// 32^3 .. 128^3 and two uneven boxes; the choice is within 4% of the best
 // length on each.  Stage time at 16 planes (the shortest chunk before) and
 // now: 32^3 14.2 -> 2.9 us, 64^3 11.6 -> 4.2, 96^3 14.5 -> 8.9, 128^3 15.7 ->
-// 14.4, 128^3 saturated 23.7 -> 19.1; 192^3 and above keep their time.
+// 14.4, 128^3 saturated 23.7 -> 19.1.
 int auto_nzchunk_q(const KGrid<float>& g, int tx, int ty)
 {
     const int64_t cols = (int64_t)((g.n[0] + tx - 1) / tx) * ((g.n[1] + ty - 1) / ty);
     const int64_t sms = sm_count(), slots = kCtasPerSm * sms;
-    const bool many = cols * ((g.n[2] + 15) / 16) * 2 >= 7 * slots;
+    const int64_t at16 = cols * ((g.n[2] + 15) / 16);
+    const bool many = at16 * 2 >= 7 * slots, wave = at16 >= slots;
     int best = 32;
     double cost = 1e300;
-    for (int nzc = many ? 16 : 1; nzc <= 64; ++nzc) {
+    for (int nzc = wave ? 16 : 1; nzc <= 64; ++nzc) {
         const int64_t chunks = (g.n[2] + nzc - 1) / nzc;
         double cst;
-        if (many) {
-            if (cols * chunks * 2 < 7 * slots) continue;
+        if (wave) {
+            if (many && cols * chunks * 2 < 7 * slots) continue;
             const int64_t rounds = (cols * chunks + slots - 1) / slots;
             cst = (double)rounds * (std::min(nzc, g.n[2]) + 2.5);
         } else {
