@@ -235,8 +235,8 @@ rkl_status rkl_super_step_s(rkl_plan *plan, double dt, int s, void *T, const voi
  * z components; ghosts copy the nearest interior cell).
  *
  * rkl_dt_hyperbolic: Eq. dt_h with lambda_d = |u_d| (a passive flow has no
- * sound speed): C_h / max_cells sum_d |u_d| / dx_d, or 0 if u = 0.  Uses one
- * stage buffer of the plan as scratch; synchronises.
+ * sound speed): C_h / max_cells sum_d |u_d| / dx_d, or 0 if u = 0.
+ * Synchronises.
  *
  * rkl_advect: one conservative first-order donor-cell step,
  * T_out = T_in - dt sum_d (F_d(c + 1/2) - F_d(c - 1/2)) / dx_d with face
@@ -392,6 +392,8 @@ rkl_status rkl_ensemble_layout(const rkl_ensemble *ens, int64_t *cell_offsets);
  * (<= 0: 32).  RKL_ERR_INVALID_ARG for persistent outside 0..3;
  * RKL_ERR_UNSUPPORTED for the row-pair tiles unless every problem is
  * periodic with fewer than 2^31 cells (the autotuner then skips them).
+ * A new ensemble starts with schedule 3 and a length chosen from its sizes
+ * (4 to 48 planes) where the row-pair tiles apply, else with 1 and 32.
  */
 rkl_status rkl_ensemble_set_schedule(rkl_ensemble *ens, int persistent, int nzchunk);
 
