@@ -859,12 +859,10 @@ rkl_status rkl_dt_hyperbolic(rkl_plan* p, const void* u, double ch, double* dt_o
     if (!u || !dt_out) return fail(p, RKL_ERR_INVALID_ARG, "null argument");
     if (!(ch > 0.0) || !std::isfinite(ch)) return fail(p, RKL_ERR_INVALID_ARG, "C_h must be finite and > 0");
     DeviceGuard dg(p->device);
-    // the rates go to a stage buffer, free between super-steps
-    cudaError_t e = launch_hyp_rate(p->cfg, p->cfg.dtype == RKL_F64 ? (const void*)&p->gd : (const void*)&p->gf, u,
-                                    p->ybuf[0], p->stream);
+    cudaError_t e = launch_rate_stats(p->cfg, p->cfg.dtype == RKL_F64 ? (const void*)&p->gd : (const void*)&p->gf, u,
+                                      p->d_partials, p->m_scal, p->stream);
     if (e != cudaSuccess) return cuda_fail(p, e, "rate launch");
-    rkl_status st = stats(p, p->ybuf[0], false, false);
-    if (st != RKL_OK) return st;
+    RKL_CK(p, cudaStreamSynchronize(p->stream));
     const double mx = p->h_scal[0];
     if (!std::isfinite(mx)) return fail(p, RKL_ERR_NONFINITE, "u holds NaN or Inf");
     *dt_out = mx > 0.0 ? ch / mx : 0.0;

@@ -74,11 +74,13 @@ cudaError_t launch_stage_col(const LaunchCfg& c, const KGrid<double>& g, const K
                              const KCoef<double>& coef, unsigned* status, cudaStream_t st);
 
 // Operator splitting: one donor-cell advection step T_out = T - dt div(u T)
-// (u: [3][ncell] cell-centred velocity), and the per-cell rate
-// sum_d |u_d| / dx_d of Eq. dt_h into lam (grid-sized scratch).
+// (u: [3][ncell] cell-centred velocity), and the statistics (as launch_stats,
+// no sum, no status word) of the per-cell rate sum_d |u_d| / dx_d of Eq. dt_h,
+// which is not stored.
 cudaError_t launch_advect(const LaunchCfg& c, const void* grid, const void* T, const void* u, void* Tout, double dt,
                           cudaStream_t st);
-cudaError_t launch_hyp_rate(const LaunchCfg& c, const void* grid, const void* u, void* lam, cudaStream_t st);
+cudaError_t launch_rate_stats(const LaunchCfg& c, const void* grid, const void* u, double* partials, double* out,
+                              cudaStream_t st);
 
 // Tiled FP32 3D stage kernel (shared-memory halo planes, z-march).
 // Returns cudaErrorNotSupported if the configuration is not covered.
