@@ -41,16 +41,6 @@ __device__ __forceinline__ void ldsm_x4(unsigned addr, unsigned& r0, unsigned& r
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
                  : "r"(addr));
 }
-__device__ __forceinline__ void ldsm_x4_t(unsigned addr, unsigned& r0, unsigned& r1, unsigned& r2, unsigned& r3)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x2_t(unsigned addr, unsigned& r0, unsigned& r1)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(addr));
-}
 __device__ __forceinline__ void ldsm_x2(unsigned addr, unsigned& r0, unsigned& r1)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(addr));
@@ -183,127 +173,6 @@ conv_kernel(const __nv_bfloat16* __restrict__ in, const __nv_bfloat16* __restric
 }
 
 // --------------------------------------------------------------------------
-// Weight gradient: dW[o][co][ci] += sum_v dz[v][co] * x[v + off(o)][ci].
-// One persistent CTA per SM walks 512-voxel tiles; per tile it stages the
-// dz tile and the x tile with its one-cell halo once and serves all 27
-// offsets from them.  The work of a tile is split into units (offset o,
-// 8-channel ci block nt), each a COUT x 8 block of dW; warp w owns units
-// w, w + 16, ... and accumulates them over all its tiles in registers,
-// then stores them to the CTA's own slice of part ([gridDim.x][27][COUT]
-// [CIN]); sum_partials adds the slices to dW in CTA order, so the result
-// does not depend on which CTA finishes first.
-// The bias gradient sum_v dz[v][co] rides along: each thread adds up one
-// channel's values of every staged dz tile (thread t: channel t % COUT),
-// and the CTA stores its per-channel sums to partb[blockIdx.x][COUT].
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(NTHR, 1)
-wgrad_kernel(const __nv_bfloat16* __restrict__ dz, const __nv_bfloat16* __restrict__ x, float* __restrict__ part,
-             float* __restrict__ partb, int D, int H, int W)
-{
-    constexpr int SZ = COUT + 8, SXC = CIN + 8;
-    constexpr int MT = COUT / 16;                       // m16 tiles over co
-    constexpr int NT = CIN / 8;                         // n8 blocks over ci
-    constexpr int NU = 27 * NT;                         // units per tile
-    constexpr int UPW = (NU + NWARP - 1) / NWARP;       // units per warp (at most)
-    static_assert(COUT % 16 == 0 && CIN % 16 == 0, "channel counts are multiples of 16");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __nv_bfloat16* sZ = reinterpret_cast<__nv_bfloat16*>(smem_raw);        // [TV][SZ]
-    __nv_bfloat16* sX = sZ + TV * SZ;                                       // [HV][SXC]
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tilesx = W / TX, tilesy = H / TY, tilesz = D / TZ;
-    const int ntiles = tilesx * tilesy * tilesz;
-
-    float bacc = 0.f;
-    float acc[UPW][MT][4];
-#pragma unroll
-    for (int i = 0; i < UPW; ++i)
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[i][mt][q] = 0.f;
-
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int bx = tile % tilesx, by = (tile / tilesx) % tilesy, bz = tile / (tilesx * tilesy);
-        const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
-        __syncthreads();
-        for (int t = tid; t < TV * (COUT / 8); t += NTHR) {
-            const int m = t / (COUT / 8), ch = t % (COUT / 8);
-            const int tx = m % TX, ty = (m / TX) % TY, tz = m / (TX * TY);
-            const int64_t gv = ((int64_t)(z0 + tz) * H + (y0 + ty)) * W + (x0 + tx);
-            cp16(smem_u32(sZ + m * SZ + ch * 8), dz + gv * COUT + ch * 8);
-        }
-        for (int t = tid; t < HV * (CIN / 8); t += NTHR) {
-            const int hv = t / (CIN / 8), ch = t % (CIN / 8);
-            const int hx = hv % HX, hy = (hv / HX) % HY, hz = hv / (HX * HY);
-            const int gz = wrapi(z0 + hz - 1, D), gy = wrapi(y0 + hy - 1, H), gx = wrapi(x0 + hx - 1, W);
-            const int64_t gv = ((int64_t)gz * H + gy) * W + gx;
-            cp16(smem_u32(sX + hv * SXC + ch * 8), x + gv * CIN + ch * 8);
-        }
-        cp_commit();
-        cp_wait_all();
-        __syncthreads();
-#pragma unroll 8
-        for (int m = tid / COUT; m < TV; m += NTHR / COUT) bacc += __bfloat162float(sZ[m * SZ + tid % COUT]);
-        for (int ks = 0; ks < TV / 16; ++ks) {
-            const int v0 = ks * 16;                      // one x-row of the tile
-            const int ty = (v0 / TX) % TY, tz = v0 / (TX * TY);
-            // A = dz^T (m = co, k = v): transpose-load rows v of sZ
-            unsigned a[MT][4];
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
-                const int q = lane >> 3, r = lane & 7;
-                const int vrow = v0 + r + 8 * (q >> 1);
-                const int cobase = mt * 16 + 8 * (q & 1);
-                ldsm_x4_t(smem_u32(sZ + vrow * SZ + cobase), a[mt][0], a[mt][1], a[mt][2], a[mt][3]);
-            }
-            // B = x shifted by the unit's offset (k = v, n = ci block)
-            const int rr = (lane & 7) + 8 * ((lane >> 3) & 1);
-            const int hvrow = ((tz + 1) * HY + (ty + 1)) * HX + rr + 1;
-#pragma unroll
-            for (int i = 0; i < UPW; ++i) {
-                const int u = warp + i * NWARP;
-                if (u < NU) {
-                    const int o = u / NT, nt = u % NT;
-                    const int dhv = ((o / 9 - 1) * HY + ((o / 3) % 3 - 1)) * HX + (o % 3 - 1);
-                    unsigned b0, b1;
-                    ldsm_x2_t(smem_u32(sX + (hvrow + dhv) * SXC + nt * 8), b0, b1);
-#pragma unroll
-                    for (int mt = 0; mt < MT; ++mt)
-                        mma16816(acc[i][mt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
-                }
-            }
-        }
-    }
-    // rows co = mt*16 + lane/4 (+8), columns ci = nt*8 + 2(lane%4) + {0, 1}
-#pragma unroll
-    for (int i = 0; i < UPW; ++i) {
-        const int u = warp + i * NWARP;
-        if (u >= NU) continue;
-        const int o = u / NT, nt = u % NT;
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int co = mt * 16 + (lane >> 2) + 8 * h;
-                const int ci = nt * 8 + 2 * (lane & 3);
-                float* dst = part + (int64_t)blockIdx.x * (27 * COUT * CIN) + ((int64_t)o * COUT + co) * CIN + ci;
-                *reinterpret_cast<float2*>(dst) = make_float2(acc[i][mt][2 * h], acc[i][mt][2 * h + 1]);
-            }
-    }
-    // the bias sums: NTHR / COUT threads per channel, added in thread order
-    __syncthreads();
-    float* red = reinterpret_cast<float*>(smem_raw);
-    red[tid] = bacc;
-    __syncthreads();
-    if (tid < COUT) {
-        float t = 0.f;
-        for (int k = 0; k < NTHR / COUT; ++k) t += red[k * COUT + tid];
-        partb[(int64_t)blockIdx.x * COUT + tid] = t;
-    }
-}
-
-// --------------------------------------------------------------------------
 // Surrogate input features (channels last, 16 channels, 6 or 9 used):
 //   T - 1, b_x, b_y, b_z, log10(kappa_par(T) / 0.01), dt/dt_expl / 100, and
 //   with F (face fluxes of T, [3][V]) fscale * F_x, F_y, F_z.
@@ -425,17 +294,6 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
     }
 }
 
-// out[i] += sum over b = 0 .. nparts - 1 of part[b][i], in that order.
-__global__ void sum_partials_kernel(const float* __restrict__ part, int nparts, int n, float* __restrict__ out)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        float t = 0.f;
-#pragma unroll 8
-        for (int b = 0; b < nparts; ++b) t += part[(int64_t)b * n + i];
-        out[i] += t;
-    }
-}
-
 }  // namespace
 
 // --------------------------------------------------------------------------
@@ -520,32 +378,6 @@ cudaError_t adam(float* p, const float* g, float* m, float* v, int n, float lr, 
     return cudaGetLastError();
 }
 
-template <int CIN, int COUT>
-static cudaError_t wgrad_t(const void* dz, const void* x, float* dW, float* db, float* part, int D, int H, int W,
-                           cudaStream_t st)
-{
-    constexpr int SZ = COUT + 8, SXC = CIN + 8;
-    const int smem = (TV * SZ + HV * SXC) * 2;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(wgrad_kernel<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    const int ntiles = (D / TZ) * (H / TY) * (W / TX);
-    const int sms = wgrad_max_ctas();
-    const int grid = ntiles < sms ? ntiles : sms;
-    float* partb = part + (size_t)grid * 27 * COUT * CIN;
-    wgrad_kernel<CIN, COUT><<<grid, NTHR, smem, st>>>(static_cast<const __nv_bfloat16*>(dz),
-                                                     static_cast<const __nv_bfloat16*>(x), part, partb, D, H, W);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    sum_partials_kernel<<<grid_for(27 * COUT * CIN), 256, 0, st>>>(part, grid, 27 * COUT * CIN, dW);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    sum_partials_kernel<<<1, 32, 0, st>>>(partb, grid, COUT, db);
-    return cudaGetLastError();
-}
-
 int wgrad_max_ctas()
 {
     static int sms = 0;
@@ -559,16 +391,6 @@ int wgrad_max_ctas()
 }
 
 size_t wgrad_workspace_floats() { return (size_t)wgrad_max_ctas() * (27 * 32 * 32 + 32); }
-
-cudaError_t conv_wgrad(int cin, int cout, const void* dz, const void* x, float* dW, float* db, float* part, int D,
-                       int H, int W, cudaStream_t st)
-{
-    if (D % TZ || H % TY || W % TX) return cudaErrorInvalidValue;
-    if (cin == 16 && cout == 32) return wgrad_t<16, 32>(dz, x, dW, db, part, D, H, W, st);
-    if (cin == 32 && cout == 32) return wgrad_t<32, 32>(dz, x, dW, db, part, D, H, W, st);
-    if (cin == 32 && cout == 16) return wgrad_t<32, 16>(dz, x, dW, db, part, D, H, W, st);
-    return cudaErrorInvalidValue;
-}
 
 
 }  // namespace conv

@@ -172,19 +172,15 @@ rkl_status backward_impl(rkl_surrogate* s, const float* target, double* loss)
     SUR_CK(s, conv::loss_and_adjoint(s->dT, target, D, H, W, (float)s->head_scale, s->inv_dx, s->r, s->d_part,
                                      kPartials, s->dG, s->stream));
     SUR_CK(s, cudaMemcpyAsync(s->h_part, s->d_part, sizeof(double) * kPartials, cudaMemcpyDeviceToHost, s->stream));
-    for (int l = 0; l < kLayers; ++l) {
-        SUR_CK(s, cudaMemsetAsync(s->gw[l], 0, sizeof(float) * wcount(l), s->stream));
-        SUR_CK(s, cudaMemsetAsync(s->gb[l], 0, sizeof(float) * kCout[l], s->stream));
-    }
     // head
     const void* dz = s->dG;
-    SUR_CK(s, conv::conv_wgrad(32, 16, dz, s->A[4], s->gw[5], s->gb[5], s->gpart, D, H, W, s->stream));
+    SUR_CK(s, conv::conv_wgrad_tc(32, 16, dz, s->A[4], s->gw[5], s->gb[5], s->gpart, D, H, W, s->d_tcst, s->stream));
     SUR_CK(s, conv_fwd(s, 16, 32, 2, dz, s->wb[5], nullptr, s->A[4], s->dZ[0]));
     int cur = 0;
     for (int l = kLayers - 2; l >= 0; --l) {
         dz = s->dZ[cur];
         const void* x = l > 0 ? s->A[l - 1] : s->X0;
-        SUR_CK(s, conv::conv_wgrad(kCin[l], 32, dz, x, s->gw[l], s->gb[l], s->gpart, D, H, W, s->stream));
+        SUR_CK(s, conv::conv_wgrad_tc(kCin[l], 32, dz, x, s->gw[l], s->gb[l], s->gpart, D, H, W, s->d_tcst, s->stream));
         if (l > 0) {
             SUR_CK(s, conv_fwd(s, 32, 32, 2, dz, s->wb[l], nullptr, s->A[l - 1], s->dZ[1 - cur]));
             cur = 1 - cur;
@@ -459,10 +455,8 @@ rkl_status rkl_sur_layer_backward_data(rkl_surrogate* s, int layer, const void* 
 rkl_status rkl_sur_layer_weight_grad(rkl_surrogate* s, int layer, const void* dz, const void* x)
 {
     if (!s || layer < 0 || layer >= kLayers || !dz || !x) return RKL_ERR_INVALID_ARG;
-    SUR_CK(s, cudaMemsetAsync(s->gw[layer], 0, sizeof(float) * wcount(layer), s->stream));
-    SUR_CK(s, cudaMemsetAsync(s->gb[layer], 0, sizeof(float) * kCout[layer], s->stream));
-    SUR_CK(s, conv::conv_wgrad(kCin[layer], kCout[layer], dz, x, s->gw[layer], s->gb[layer], s->gpart, s->D, s->H,
-                               s->W, s->stream));
+    SUR_CK(s, conv::conv_wgrad_tc(kCin[layer], kCout[layer], dz, x, s->gw[layer], s->gb[layer], s->gpart, s->D,
+                                  s->H, s->W, s->d_tcst, s->stream));
     return RKL_OK;
 }
 
