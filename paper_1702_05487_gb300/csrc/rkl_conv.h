@@ -35,8 +35,7 @@ cudaError_t features(const float* T, const float* b, int64_t V, float kappa0, in
 cudaError_t head_div(const float* G, int D, int H, int W, float tau, const float inv_dx[3], float* dT,
                      cudaStream_t st);
 cudaError_t loss_and_adjoint(const float* dT, const float* target, int D, int H, int W, float tau,
-                             const float inv_dx[3], float* r, double* partial, int npartial, void* dG,
-                             cudaStream_t st);
+                             const float inv_dx[3], double* partial, int npartial, void* dG, cudaStream_t st);
 cudaError_t pack_weights(const float* w, int cout, int cin, void* wf, void* wb, cudaStream_t st);
 cudaError_t adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float eps, int t,
                  cudaStream_t st);

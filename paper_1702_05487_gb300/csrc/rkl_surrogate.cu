@@ -106,7 +106,6 @@ struct rkl_surrogate {
     void* A[kLayers - 1] = {};     // bf16 [V][32]
     float* G = nullptr;            // f32 [V][16]
     float* dT = nullptr;           // f32 [V]
-    float* r = nullptr;            // f32 [V]
     void* dG = nullptr;            // bf16 [V][16]
     void* dZ[2] = {};              // bf16 [V][32]
     float* gpart = nullptr;        // per-CTA partial weight / bias gradients (fixed-order sums)
@@ -169,7 +168,7 @@ rkl_status forward_impl(rkl_surrogate* s, double head_scale)
 rkl_status backward_impl(rkl_surrogate* s, const float* target, double* loss)
 {
     const int D = s->D, H = s->H, W = s->W;
-    SUR_CK(s, conv::loss_and_adjoint(s->dT, target, D, H, W, (float)s->head_scale, s->inv_dx, s->r, s->d_part,
+    SUR_CK(s, conv::loss_and_adjoint(s->dT, target, D, H, W, (float)s->head_scale, s->inv_dx, s->d_part,
                                      kPartials, s->dG, s->stream));
     SUR_CK(s, cudaMemcpyAsync(s->h_part, s->d_part, sizeof(double) * kPartials, cudaMemcpyDeviceToHost, s->stream));
     // head
@@ -256,7 +255,6 @@ rkl_status rkl_sur_create(int D, int H, int W, const double* dx, void* cuda_stre
         if ((c = cudaMalloc(&s->A[l], (size_t)V * 32 * 2)) != cudaSuccess) return bail(c, "activations");
     if ((c = cudaMalloc(&s->G, (size_t)V * 16 * 4)) != cudaSuccess) return bail(c, "head");
     if ((c = cudaMalloc(&s->dT, (size_t)V * 4)) != cudaSuccess) return bail(c, "dT");
-    if ((c = cudaMalloc(&s->r, (size_t)V * 4)) != cudaSuccess) return bail(c, "r");
     if ((c = cudaMalloc(&s->dG, (size_t)V * 16 * 2)) != cudaSuccess) return bail(c, "dG");
     for (int k = 0; k < 2; ++k)
         if ((c = cudaMalloc(&s->dZ[k], (size_t)V * 32 * 2)) != cudaSuccess) return bail(c, "dZ");
@@ -288,7 +286,7 @@ rkl_status rkl_sur_destroy(rkl_surrogate* s)
     }
     cudaFree(s->X0);
     for (int l = 0; l < kLayers - 1; ++l) cudaFree(s->A[l]);
-    cudaFree(s->G); cudaFree(s->dT); cudaFree(s->r); cudaFree(s->dG);
+    cudaFree(s->G); cudaFree(s->dT); cudaFree(s->dG);
     cudaFree(s->dZ[0]); cudaFree(s->dZ[1]);
     cudaFree(s->Yp); cudaFree(s->M0); cudaFree(s->Mp); cudaFree(s->F3);
     cudaFree(s->d_part);
