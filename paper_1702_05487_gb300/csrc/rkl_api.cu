@@ -243,7 +243,7 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
                                 p->variant == 4 ? 3 : (p->variant == 9 ? 6 : 2), st, p->variant == 6,
                                 p->variant == 7, p->variant == 8);
         else if (p->colok && p->variant != 1 && p->variant != 2)
-            e = launch_stage_col(p->cfg, p->gf, p->pf, io, cf, p->d_status, st);
+            e = launch_stage_plane(p->cfg, p->gf, p->pf, io, cf, p->d_status, st);
         else if (p->fast && al && (p->variant == 0 || p->variant == 2))
             e = launch_stage_fast(p->cfg, p->gf, p->pf, io, cf, p->d_status, st);
         else

@@ -1,5 +1,5 @@
-// Column-march stage kernels (rkl_col.cuh), FP32 instances, and the rule for
-// the grids they take.
+// Column-march stage kernels (rkl_col.cuh) and the rule for the grids they
+// take.
 #include "rkl_col.cuh"
 
 namespace rkl {
@@ -28,11 +28,11 @@ bool col_stage_supported(int dtype, int ndim, const int n[3], int64_t plane)
     return ndim == 3 && dtype == 1 && plane < ((int64_t)1 << 31) && n[1] <= 8 * 65535 && n[2] <= 65535;
 }
 
-cudaError_t launch_stage_col(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
-                             const KCoef<float>& coef, unsigned* status, cudaStream_t st)
+cudaError_t launch_stage_col(const LaunchCfg& c, const KGrid<double>& g, const KPhys<double>& p, const StageIO& io,
+                             const KCoef<double>& coef, unsigned* status, cudaStream_t st)
 {
     if (!col_stage_supported(c.dtype, c.ndim, g.n, g.plane)) return cudaErrorNotSupported;
-    return col::launch<float>(c, g, p, io, coef, status, st);
+    return col::launch<double>(c, g, p, io, coef, status, st);
 }
 
 }  // namespace rkl

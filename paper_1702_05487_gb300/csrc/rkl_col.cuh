@@ -1,6 +1,6 @@
-// Column-march stage kernels of the RKL2 conduction super-step: FP64 3D grids
-// and 2D grids of either type (the packed FP32 tile kernels take the rest),
-// periodic or Dirichlet, limiter at any floor.  One thread per cell column,
+// Column-march stage kernels of the RKL2 conduction super-step for FP64 grids,
+// 3D and 2D (rkl_plane.cu has the packed FP32 form of the 2D one), periodic or
+// Dirichlet, limiter at any floor.  One thread per cell column,
 // marching along the slowest axis; every face is evaluated once:
 //
 //   3D  eight warps of a block cover LPR columns x 256 / LPR rows of a plane
@@ -21,8 +21,7 @@
 // and integer checks of the result: about 95 FP64 operations per cell and
 // stage against about 305 in the generic kernel, which evaluates both faces
 // of every axis.  112 x 96 x 80 FP64 stage (Spitzer): generic 419 us, this
-// kernel 176 us.  In 2D it is instruction issue and latency: 1530 x 1071
-// FP32 saturated stage 92 -> 17 us, 100 x 100 FP64 Dirichlet 8.2 -> 3.2 us.
+// kernel 176 us; 100 x 100 Dirichlet 8.2 -> 3.1 us.
 #pragma once
 
 #include <algorithm>
@@ -523,15 +522,13 @@ template <typename R, bool SP, bool SAT, bool LIM, bool CUBE>
 cudaError_t launch_nd(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, const Args<R>& a, const KCoef<R>& cf,
                       unsigned* status, cudaStream_t st, bool chained)
 {
-    if constexpr (sizeof(R) == 8) {
-        if (c.ndim == 3) {
-            const int lpr = lanes_per_row(g.n[0], g.n[1]), rows = NW * 32 / lpr;
-            const int bx = (g.n[0] + lpr - 1) / lpr, by = (g.n[1] + rows - 1) / rows;
-            const int nzc = chunk3((int64_t)bx * by, g.n[2]);
-            const dim3 grid(bx, by, (g.n[2] + nzc - 1) / nzc);
-            return launch_chained(col3_kernel<R, SP, SAT, LIM, CUBE>, grid, NT, 0, st, chained, g, p, a, cf, status, nzc,
-                                  lpr);
-        }
+    if (c.ndim == 3) {
+        const int lpr = lanes_per_row(g.n[0], g.n[1]), rows = NW * 32 / lpr;
+        const int bx = (g.n[0] + lpr - 1) / lpr, by = (g.n[1] + rows - 1) / rows;
+        const int nzc = chunk3((int64_t)bx * by, g.n[2]);
+        const dim3 grid(bx, by, (g.n[2] + nzc - 1) / nzc);
+        return launch_chained(col3_kernel<R, SP, SAT, LIM, CUBE>, grid, NT, 0, st, chained, g, p, a, cf, status, nzc,
+                              lpr);
     }
     const int ntx = (g.n[0] + 30) / 31;
     // rows per warp: about 32 warps per SM, at most 32 rows
@@ -556,13 +553,19 @@ cudaError_t launch_form(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p
 }
 
 template <typename R>
+Args<R> stage_args(const StageIO& io)
+{
+    return Args<R>{static_cast<const R*>(io.mode == 1 ? io.Y0 : io.Yjm1), static_cast<const R*>(io.b),
+                   static_cast<const R*>(io.Y0), static_cast<const R*>(io.Yjm2), static_cast<const R*>(io.MY0),
+                   io.mode == 1 ? static_cast<R*>(io.MY0) : nullptr, static_cast<R*>(io.Yj),
+                   static_cast<const R*>(io.coef_tab), io.j, io.mode};
+}
+
+template <typename R>
 cudaError_t launch(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, const StageIO& io, const KCoef<R>& cf,
                    unsigned* status, cudaStream_t st)
 {
-    const Args<R> a{static_cast<const R*>(io.mode == 1 ? io.Y0 : io.Yjm1), static_cast<const R*>(io.b),
-                    static_cast<const R*>(io.Y0), static_cast<const R*>(io.Yjm2), static_cast<const R*>(io.MY0),
-                    io.mode == 1 ? static_cast<R*>(io.MY0) : nullptr, static_cast<R*>(io.Yj),
-                    static_cast<const R*>(io.coef_tab), io.j, io.mode};
+    const Args<R> a = stage_args<R>(io);
     if (c.spitzer)
         return c.saturate ? launch_form<R, true, true>(c, g, p, a, cf, status, st, io.chained)
                           : launch_form<R, true, false>(c, g, p, a, cf, status, st, io.chained);

@@ -65,13 +65,14 @@ cudaError_t launch_stage_generic(const LaunchCfg& c, const void* grid, const voi
 cudaError_t launch_flux_generic(const LaunchCfg& c, const void* grid, const void* phys,
                                 const void* T, const void* b, void* F[3], cudaStream_t st);
 
-// Column-march stage kernels: 2D grids of either type and FP64 3D grids, any
-// width, either boundary, limiter at any floor; each face evaluated once.
+// Column-march stage kernels: 2D grids (FP64, and FP32 in packed pairs) and
+// FP64 3D grids, any width, either boundary, limiter at any floor (FP32: at
+// every face); each face evaluated once.
 bool col_stage_supported(int dtype, int ndim, const int n[3], int64_t plane);
-cudaError_t launch_stage_col(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
-                             const KCoef<float>& coef, unsigned* status, cudaStream_t st);
 cudaError_t launch_stage_col(const LaunchCfg& c, const KGrid<double>& g, const KPhys<double>& p, const StageIO& io,
                              const KCoef<double>& coef, unsigned* status, cudaStream_t st);
+cudaError_t launch_stage_plane(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
+                               const KCoef<float>& coef, unsigned* status, cudaStream_t st);
 
 // Operator splitting: one donor-cell advection step T_out = T - dt div(u T)
 // (u: [3][ncell] cell-centred velocity), and the statistics (as launch_stats,
