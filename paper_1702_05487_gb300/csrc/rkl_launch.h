@@ -123,7 +123,8 @@ cudaError_t launch_stage_xq(const LaunchCfg& c, const KGrid<float>& g, const KPh
                             int txw = 64);
 
 // Row-pair FP32 3D stage kernel for any width and either boundary (rows
-// copied in 4-byte pieces, 64-column tiles): no limiter or the limiter at
+// copied in 4-byte pieces, or in 16-byte chunks on Dirichlet grids with nx %
+// 4 == 0; 64-column tiles): no limiter or the limiter at
 // every face, fewer than 2^31 cells, 16-byte aligned arrays; nzchunk <= 0
 // picks the chunk length.
 bool xg_stage_supported(const LaunchCfg& c, const KGrid<float>& g);

@@ -11,11 +11,11 @@ cudaError_t launch_q_gen_lim(bool sp, bool sat, int mode, const KGrid<float>& g,
                              cudaStream_t st, bool chained)
 {
     if (sp) {
-        if (sat) return launch_q_mode<true, true, 64, false, true, true>(mode, g, p, a, cf, status, nzchunk, st, chained);
-        return launch_q_mode<true, false, 64, false, true, true>(mode, g, p, a, cf, status, nzchunk, st, chained);
+        if (sat) return launch_q_mode<true, true, 64, false, true, Q_GEN>(mode, g, p, a, cf, status, nzchunk, st, chained);
+        return launch_q_mode<true, false, 64, false, true, Q_GEN>(mode, g, p, a, cf, status, nzchunk, st, chained);
     }
-    if (sat) return launch_q_mode<false, true, 64, false, true, true>(mode, g, p, a, cf, status, nzchunk, st, chained);
-    return launch_q_mode<false, false, 64, false, true, true>(mode, g, p, a, cf, status, nzchunk, st, chained);
+    if (sat) return launch_q_mode<false, true, 64, false, true, Q_GEN>(mode, g, p, a, cf, status, nzchunk, st, chained);
+    return launch_q_mode<false, false, 64, false, true, Q_GEN>(mode, g, p, a, cf, status, nzchunk, st, chained);
 }
 
 }  // namespace xq

@@ -177,6 +177,9 @@ cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPh
     const x2::FastArgs a = x2_args(io);
     int nzc = nzchunk > 0 ? nzchunk : xq::auto_nzchunk_q(g, 64, xq::SmemQ<64>::TY);
     nzc = std::max(nzc, (g.n[2] + 65534) / 65535);      // the grid's z limit
+    if (g.bc == 1 && g.n[0] % 4 == 0)
+        return (c.limiter ? xq::launch_q_dir_lim : xq::launch_q_dir)(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a,
+                                                                     coef, status, nzc, st, io.chained);
     if (c.limiter) return xq::launch_q_gen_lim(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st, io.chained);
     return xq::launch_q_gen(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st, io.chained);
 }

@@ -32,7 +32,8 @@
 // same operation on the same operands, in the same order, as in the
 // paired-cell kernel (rkl_x2_tile.cuh), so the two kernels write the same
 // bits.  Grids with fewer than 2^31 cells: periodic with nx % 4 == 0, or
-// (GEN builds) any width and either boundary.  A GEN build copies rows in
+// (GEN builds) any width and either boundary, or (DIR builds) Dirichlet with
+// nx % 4 == 0, which keep the 16-byte chunks.  A GEN build copies rows in
 // 4-byte pieces, one cell per lane, because 16-byte chunks of a row start
 // aligned in global memory only if nx % 4 == 0: a warp's copy of 32 cells is
 // then one or two 128-byte lines, so the shared-memory and L1 traffic stay
@@ -40,7 +41,8 @@
 // thread and plane instead of 9).  Each lane's wrapped or clamped column and
 // row offsets are fixed per tile; Dirichlet ghosts of T are stored, not
 // copied.  201 x 150 x 99 stage: 138 us (one-cell tiled kernel) ->
-// 38 us; Dirichlet 192 x 128 x 96, constant kappa: 29 (paired-cell) -> 23 us.
+// 38 us.  Dirichlet 192 x 128 x 96, constant kappa: paired-cell 29
+// us, GEN 22, DIR 16.
 #pragma once
 
 #include <algorithm>
@@ -220,12 +222,32 @@ __device__ __forceinline__ GenPos<SM> gen_pos(const KGrid<float>& g, int tid, in
     return n;
 }
 
-template <bool SP, bool SAT, int MODE, int TXW, bool KP0 = false, bool LIM = false, bool GEN = false>
+// Copy positions of a DIR build (Dirichlet, nx % 4 == 0): as tb_pos, but rows
+// and chunks past the edge are ghosts, flagged in the low bits of dst: T is
+// stored, and of a b chunk past the x edge only the cell beside the grid is
+// used, which repeats the edge cell (one 4-byte copy).
+enum : unsigned { PF_GHOST = 1u, PF_LEFT = 2u, PF_RIGHT = 4u, PF_ALL = 15u };
+template <class SM>
+__device__ __forceinline__ Pos dir_pos(const KGrid<float>& g, int t, int i0, int j0)
+{
+    if (t >= SM::kPos) return Pos{0u, ~0u};
+    const int row = t / SM::CPR - 1, cc = (t % SM::CPR) * 4 - 4;
+    const int gy = j0 + row, gx = i0 + cc;
+    const bool xl = gx < 0, xr = gx >= g.n[0];
+    const unsigned f = (xl || xr || gy < 0 || gy >= g.n[1] ? PF_GHOST : 0u) | (xl ? PF_LEFT : 0u) | (xr ? PF_RIGHT : 0u);
+    const int sx = xl ? 0 : (xr ? g.n[0] - 1 : gx);
+    return Pos{(unsigned)clampi(gy, g.n[1]) * (unsigned)g.n[0] + (unsigned)sx, (unsigned)(SM::off(row, cc) * 4) | f};
+}
+
+enum { Q_PERIODIC = 0, Q_GEN = 1, Q_DIR = 2 };      // how a tile's bundles are copied
+
+template <bool SP, bool SAT, int MODE, int TXW, bool KP0 = false, bool LIM = false, int EDGE = Q_PERIODIC>
 __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, const KPhys<float>& p,
                                        const x2::FastArgs& a, KCoef<float> cf, unsigned* status, int i0, int j0,
                                        int z0, int nzc)
 {
     using Smem = SmemQ<TXW>;
+    constexpr bool GEN = EDGE == Q_GEN, DIR = EDGE == Q_DIR;
     constexpr int TX = Smem::TX, TY = Smem::TY, LPR = Smem::LPR, SEGS = Smem::SEGS;
     constexpr int PLANE = Smem::PLANE;
     const int tid = threadIdx.x;
@@ -247,8 +269,8 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     if (GEN) {
         gp = gen_pos<Smem>(g, tid, i0, j0);
     } else {
-        p0 = tb_pos<Smem>(g, tid, i0, j0);
-        p1 = tb_pos<Smem>(g, tid + NTHREADS, i0, j0);
+        p0 = DIR ? dir_pos<Smem>(g, tid, i0, j0) : tb_pos<Smem>(g, tid, i0, j0);
+        p1 = DIR ? dir_pos<Smem>(g, tid + NTHREADS, i0, j0) : tb_pos<Smem>(g, tid + NTHREADS, i0, j0);
         if (MODE == 2) py = y_pos<Smem>(g, tid, i0, j0);
     }
     const float* bxp = a.b;
@@ -265,7 +287,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     // T and b of plane k, and (stages j >= 2) the Y bundle of plane k - 1
     auto load = [&](int k) {
         int kz = z0 + k;
-        const bool zg = GEN && g.bc == 1 && (kz < 0 || kz >= nz);
+        const bool zg = (DIR || (GEN && g.bc == 1)) && (kz < 0 || kz >= nz);
         if (zg) kz = kz < 0 ? 0 : nz - 1;       // Dirichlet: ghosts, b of the nearest plane
         kz += kz < 0 ? nz : 0;                  // periodic: wrap the plane index
         kz -= kz >= nz ? nz : 0;
@@ -308,20 +330,31 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
             }
             return;
         }
-        {
-            const unsigned x = p0.src + pt;
-            cp16(ts + p0.dst, a.Tin + x);
-            cp16(bs + p0.dst, bxp + x);
-            cp16(bs + PLANE * 4 + p0.dst, byp + x);
-            cp16(bs + 2 * PLANE * 4 + p0.dst, bzp + x);
-        }
-        if (p1.dst != ~0u) {
-            const unsigned x = p1.src + pt;
-            cp16(ts + p1.dst, a.Tin + x);
-            cp16(bs + p1.dst, bxp + x);
-            cp16(bs + PLANE * 4 + p1.dst, byp + x);
-            cp16(bs + 2 * PLANE * 4 + p1.dst, bzp + x);
-        }
+        auto copy = [&](const Pos& p) {
+            const unsigned x = p.src + pt;
+            if (DIR && ((p.dst & PF_ALL) || zg)) {
+                const unsigned d = p.dst & ~PF_ALL;
+                if (zg || (p.dst & PF_GHOST)) x2::st4(ts + d, g.bcv);
+                else cp16(ts + d, a.Tin + x);
+                if (p.dst & (PF_LEFT | PF_RIGHT)) {
+                    const unsigned e = bs + d + ((p.dst & PF_LEFT) ? 12u : 0u);
+                    cp4(e, bxp + x);
+                    cp4(e + PLANE * 4, byp + x);
+                    cp4(e + 2 * PLANE * 4, bzp + x);
+                } else {
+                    cp16(bs + d, bxp + x);
+                    cp16(bs + PLANE * 4 + d, byp + x);
+                    cp16(bs + 2 * PLANE * 4 + d, bzp + x);
+                }
+                return;
+            }
+            cp16(ts + p.dst, a.Tin + x);
+            cp16(bs + p.dst, bxp + x);
+            cp16(bs + PLANE * 4 + p.dst, byp + x);
+            cp16(bs + 2 * PLANE * 4 + p.dst, bzp + x);
+        };
+        copy(p0);
+        if (p1.dst != ~0u) copy(p1);
         if (MODE == 2 && k >= 1 && py.dst != ~0u) {
             // plane k - 1 lies inside the chunk, so inside the grid
             const unsigned x = py.src + (unsigned)(z0 + k - 1) * plane;
@@ -547,18 +580,18 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     __syncthreads();
 }
 
-template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM, bool GEN>
+template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM, int EDGE>
 __global__ void __launch_bounds__(NTHREADS, kCtasPerSm)
 stage_q_kernel(KGrid<float> g, KPhys<float> p, x2::FastArgs a, KCoef<float> cf, unsigned* status, int nzchunk)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     SmemQ<TXW>& sm = *reinterpret_cast<SmemQ<TXW>*>(smem_raw);
     const int z0 = blockIdx.z * nzchunk;
-    tile_q<SP, SAT, MODE, TXW, KP0, LIM, GEN>(sm, g, p, a, cf, status, blockIdx.x * SmemQ<TXW>::TX, blockIdx.y * SmemQ<TXW>::TY,
+    tile_q<SP, SAT, MODE, TXW, KP0, LIM, EDGE>(sm, g, p, a, cf, status, blockIdx.x * SmemQ<TXW>::TX, blockIdx.y * SmemQ<TXW>::TY,
                                z0, min(nzchunk, g.n[2] - z0));
 }
 
-template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM, bool GEN>
+template <bool SP, bool SAT, int MODE, int TXW, bool KP0, bool LIM, int EDGE>
 cudaError_t launch_q(const KGrid<float>& g, const KPhys<float>& p, const x2::FastArgs& a, const KCoef<float>& cf,
                      unsigned* status, int nzchunk, cudaStream_t st, bool chained)
 {
@@ -566,23 +599,23 @@ cudaError_t launch_q(const KGrid<float>& g, const KPhys<float>& p, const x2::Fas
     const int smem = (int)sizeof(SM);
     static bool attr_set = false;       // the attribute is per function, set once
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM, GEN>,
+        cudaError_t e = cudaFuncSetAttribute(stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM, EDGE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     const dim3 grid((g.n[0] + SM::TX - 1) / SM::TX, (g.n[1] + SM::TY - 1) / SM::TY, (g.n[2] + nzchunk - 1) / nzchunk);
-    return launch_chained(stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM, GEN>, grid, NTHREADS, smem, st, chained, g, p, a,
+    return launch_chained(stage_q_kernel<SP, SAT, MODE, TXW, KP0, LIM, EDGE>, grid, NTHREADS, smem, st, chained, g, p, a,
                           cf, status, nzchunk);
 }
 
-template <bool SP, bool SAT, int TXW, bool KP0, bool LIM = false, bool GEN = false>
+template <bool SP, bool SAT, int TXW, bool KP0, bool LIM = false, int EDGE = Q_PERIODIC>
 cudaError_t launch_q_mode(int mode, const KGrid<float>& g, const KPhys<float>& p, const x2::FastArgs& a,
                           const KCoef<float>& cf, unsigned* status, int nzchunk, cudaStream_t st, bool chained)
 {
-    if (mode == 0) return launch_q<SP, SAT, 0, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st, chained);
-    if (mode == 1) return launch_q<SP, SAT, 1, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st, chained);
-    return launch_q<SP, SAT, 2, TXW, KP0, LIM, GEN>(g, p, a, cf, status, nzchunk, st, chained);
+    if (mode == 0) return launch_q<SP, SAT, 0, TXW, KP0, LIM, EDGE>(g, p, a, cf, status, nzchunk, st, chained);
+    if (mode == 1) return launch_q<SP, SAT, 1, TXW, KP0, LIM, EDGE>(g, p, a, cf, status, nzchunk, st, chained);
+    return launch_q<SP, SAT, 2, TXW, KP0, LIM, EDGE>(g, p, a, cf, status, nzchunk, st, chained);
 }
 
 // Launches of the builds compiled in rkl_xq_sat.cu (saturated flux; kp0:
@@ -594,12 +627,19 @@ cudaError_t launch_q_sat(bool sp, bool kp0, int txw, int mode, const KGrid<float
 cudaError_t launch_q_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
                          cudaStream_t st, bool chained);
-// GEN builds (rkl_xg.cu: classical and saturated flux, rkl_xg_lim.cu: MC
-// limiter; 64-column tiles).
+// Builds for other grids, 64-column tiles, with the plain or (_lim) the
+// MC-limited gradients: GEN (rkl_xg.cu, rkl_xg_lim.cu) and DIR (rkl_xd.cu,
+// rkl_xd_lim.cu).
 cudaError_t launch_q_gen(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
                          cudaStream_t st, bool chained);
 cudaError_t launch_q_gen_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
+                             const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
+                             cudaStream_t st, bool chained);
+cudaError_t launch_q_dir(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
+                         const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
+                         cudaStream_t st, bool chained);
+cudaError_t launch_q_dir_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                              const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
                              cudaStream_t st, bool chained);
 

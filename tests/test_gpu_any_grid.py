@@ -1,6 +1,6 @@
 """The kernels of the automatic choice off the packed tiles' grids -- the
-row-pair kernel's builds for any width and either boundary (FP32 3D) and the
-column-march kernels (FP64 3D, 2D) -- against the FP64 oracle at the edges of
+row-pair kernel's builds for any width and either boundary (FP32 3D), the
+column-march kernels (FP64 3D, 2D) and the packed 2D kernel -- against the FP64 oracle at the edges of
 their tiles: one cell, widths and heights one below, at and one above a tile,
 odd widths, single planes; cubic and non-cubic cells, both boundaries,
 saturated (both readings of c_iso) and MC-limited fluxes."""
@@ -21,7 +21,8 @@ PHYS = {
     "sat_upwind": dict(kappa_model="spitzer", kappa_par0=0.01, saturate=True, phi=0.05, sat_upwind=True),
     "mc": dict(SPITZ, limiter="mc"),
 }
-SHAPES_F32 = [(1, 1, 3), (2, 1, 1), (3, 9, 5), (5, 8, 63), (4, 7, 65), (20, 17, 66), (3, 16, 130), (9, 2, 129)]
+SHAPES_F32 = [(1, 1, 3), (2, 1, 1), (3, 9, 5), (5, 8, 63), (4, 7, 65), (20, 17, 66), (3, 16, 130), (9, 2, 129),
+              (3, 1, 4), (5, 8, 64), (12, 9, 68), (4, 17, 128)]
 SHAPES_F64 = [(1, 1, 1), (2, 1, 3), (3, 9, 5), (4, 33, 17), (20, 16, 31), (6, 8, 33), (3, 40, 9)]
 SHAPES_2D = [(1, 1), (2, 3), (5, 30), (7, 31), (40, 32), (9, 62), (130, 63)]
 
