@@ -157,7 +157,9 @@ rkl_status rkl_coeffs_method(int method, int s, double sts_nu, double *mu, doubl
  * Create a plan for one grid and physics on a CUDA stream (cudaStream_t
  * passed as void*; NULL is the legacy default stream).  The plan allocates
  * its own device workspace: three stage buffers, M(Y_0), reduction scratch
- * (4 grid arrays plus a few KB) and caches one CUDA graph per distinct
+ * (4 grid arrays plus a few KB; FP32 3D plans whose width is not a multiple of
+ * four also hold copies of T and b with padded rows, where memory allows) and
+ * caches one CUDA graph per distinct
  * (s, T, b) triple used by rkl_super_step.  The device current at creation
  * is used for every later call.  Writes *out; destroy with
  * rkl_plan_destroy.
@@ -251,9 +253,10 @@ rkl_status rkl_advect(rkl_plan *plan, double dt, const void *u, const void *T_in
 rkl_status rkl_energy(rkl_plan *plan, const void *T, double *E_out);
 
 /*
- * Kernel choice for the stage launches of this plan: 0 = automatic (the
- * row-pair kernel where it applies, else the paired-cell kernel, else the
- * tiled kernel, else the generic kernel), 1 = the generic one-thread-per-cell kernel, 2 = the
+ * Kernel choice for the stage launches of this plan: 0 = automatic (FP32 3D:
+ * the row-pair kernel in the build for the grid's width and boundary, or the
+ * tiled kernel for a limiter with a finite floor; 2D and FP64: the
+ * column-march kernels; else the generic kernel), 1 = the generic one-thread-per-cell kernel, 2 = the
  * tiled FP32 3D kernel (32 x 8 tiles, one cell per thread), 3 and 4 = the
  * paired-cell FP32 3D kernel (64 x 4 tiles, two cells per thread in packed
  * f32x2 arithmetic; needs nx % 4 == 0) built for 20 (variant 3) or 24

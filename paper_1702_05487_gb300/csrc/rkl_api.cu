@@ -54,6 +54,13 @@ struct rkl_plan {
     bool pairok = false;               // two-stage kernel applies to the grid
     bool xqok = false;                 // row-pair kernel applies to the grid
     bool xgok = false;                 // row-pair kernel for any width and boundary applies
+    // FP32 3D widths that are not a multiple of four: super-steps run on
+    // row-padded arrays (the plan's buffers and copies of T and b), whose rows
+    // start 16-byte aligned
+    bool padok = false;
+    KGrid<float> gpad{};
+    void* padT = nullptr;
+    void* padb = nullptr;
     bool colok = false;                // column-march kernel applies to the grid
     void* my0 = nullptr;
     double* d_partials = nullptr;
@@ -232,7 +239,9 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
         KCoef<float> cf{(float)mu, (float)nu, (float)mt, (float)gt};
         bool al = aligned16(io.Y0) && aligned16(io.MY0) && aligned16(io.Yjm1) && aligned16(io.Yjm2) &&
                   aligned16(io.Yj) && aligned16(io.b);
-        if ((p->variant == 0 || p->variant == 10 || p->variant == 11) && p->xqok && al) {
+        if (io.padded)
+            e = launch_stage_xp(p->cfg, p->gpad, p->pf, io, cf, p->d_status, p->nzchunk, st);
+        else if ((p->variant == 0 || p->variant == 10 || p->variant == 11) && p->xqok && al) {
             const bool narrow = p->variant == 11 || (p->variant == 0 && narrow_tiles(p->gf.n[0]));
             e = launch_stage_xq(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk, st, narrow ? 32 : 64);
         }
@@ -260,13 +269,20 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
 // Enqueue the s stages of one super-step reading coefficients from the
 // plan's device table (stage j at d_coef[4 j]).  Y0 = T; the last stage
 // writes T (each cell reads its own Y0 before overwriting it).
-rkl_status enqueue_stages(rkl_plan* p, int s, void* T, const void* b, bool with_events, cudaStream_t cs)
+rkl_status enqueue_stages(rkl_plan* p, int s, void* Tuser, const void* buser, bool with_events, cudaStream_t cs)
 {
+    // 201 x 150 x 99: the copies cost 20 us, a stage on padded rows takes 31 us,
+    // on the caller's 38 us, so they pay from four stages on
+    const bool padded = p->padok && p->variant == 0 && s >= 4;
+    void* T = padded ? p->padT : Tuser;
+    const void* b = padded ? p->padb : buser;
+    if (padded) RKL_CK(p, launch_pack_rows(p->gpad, Tuser, buser, p->padT, p->padb, cs));
     // stages of a few microseconds start behind one another (not across the
     // timing events); from 2^21 cells on it gains nothing (201 x 150 x 99 and
     // 192 x 128 x 96: the same, 256^3: under 1% slower)
     const bool chained = !with_events && p->ncell < ((int64_t)1 << 21);
     StageIO io{};
+    io.padded = padded;
     io.b = b;
     io.coef_tab = p->d_coef;
     io.Y0 = T;
@@ -277,7 +293,8 @@ rkl_status enqueue_stages(rkl_plan* p, int s, void* T, const void* b, bool with_
     rkl_status st = launch_stage(p, io, 0, 0, 0, 0, cs);
     if (st != RKL_OK) return st;
     if (s == 1) {                      // single forward-Euler stage (RKL1, AAG-STS)
-        RKL_CK(p, cudaMemcpyAsync(T, p->ybuf[0], (size_t)p->ncell * p->esize, cudaMemcpyDeviceToDevice, cs));
+        if (padded) RKL_CK(p, launch_unpack_rows(p->gpad, p->ybuf[0], Tuser, cs));
+        else RKL_CK(p, cudaMemcpyAsync(T, p->ybuf[0], (size_t)p->ncell * p->esize, cudaMemcpyDeviceToDevice, cs));
         return RKL_OK;
     }
     if (with_events) RKL_CK(p, cudaEventRecordWithFlags(p->ev_a, cs, cudaEventRecordExternal));
@@ -331,6 +348,7 @@ rkl_status enqueue_stages(rkl_plan* p, int s, void* T, const void* b, bool with_
     }
     for (int j = 2; j <= s; ++j) {
         StageIO q{};
+        q.padded = padded;
         q.chained = chained;
         q.b = b;
         q.coef_tab = p->d_coef;
@@ -345,6 +363,7 @@ rkl_status enqueue_stages(rkl_plan* p, int s, void* T, const void* b, bool with_
         if (st != RKL_OK) return st;
     }
     if (with_events) RKL_CK(p, cudaEventRecordWithFlags(p->ev_b, cs, cudaEventRecordExternal));
+    if (padded) RKL_CK(p, launch_unpack_rows(p->gpad, T, Tuser, cs));
     return RKL_OK;
 }
 
@@ -635,6 +654,17 @@ rkl_status rkl_plan_create(const rkl_grid* grid, const rkl_phys* phys, void* cud
     p->colok = col_stage_supported(g.dtype, g.ndim, p->gf.n, p->gf.plane) &&
                (g.dtype == RKL_F64 || !p->cfg.limiter || p->cfg.lim_all);
 
+    size_t cells = (size_t)ncell;
+    if (p->xgok && g.n[0] % 4 != 0) {
+        KGrid<float>& q = p->gpad;
+        q = p->gf;
+        q.pitch = (int)((g.n[0] + 3) / 4 * 4);
+        q.plane = (int64_t)q.pitch * g.n[1];
+        q.ncell = q.plane * g.n[2];
+        p->padok = xg_stage_supported(p->cfg, q);
+        if (p->padok) cells = (size_t)q.ncell;
+    }
+
     rkl_plan* P = p;
     auto bail = [&](cudaError_t e, const char* where) {
         std::string m = std::string(where) + ": " + cudaGetErrorString(e);
@@ -645,10 +675,17 @@ rkl_status rkl_plan_create(const rkl_grid* grid, const rkl_phys* phys, void* cud
     if ((e = cudaGetDevice(&p->device)) != cudaSuccess) return bail(e, "cudaGetDevice");
     if ((e = cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking)) != cudaSuccess)
         return bail(e, "cudaStreamCreate");
-    size_t bytes = (size_t)ncell * p->esize;
+    size_t bytes = cells * p->esize;
     for (int k = 0; k < 3; ++k)
         if ((e = cudaMalloc(&p->ybuf[k], bytes)) != cudaSuccess) return bail(e, "cudaMalloc(stage buffer)");
     if ((e = cudaMalloc(&p->my0, bytes)) != cudaSuccess) return bail(e, "cudaMalloc(MY0)");
+    if (p->padok && (cudaMalloc(&p->padT, bytes) != cudaSuccess || cudaMalloc(&p->padb, 3 * bytes) != cudaSuccess)) {
+        // no room for the copies: the stages read the caller's rows
+        cudaGetLastError();
+        cudaFree(p->padT);
+        p->padT = nullptr;
+        p->padok = false;
+    }
     // partials of the statistics pass, then its block ticket counter (zeroed)
     if ((e = cudaMalloc(&p->d_partials, sizeof(double) * (3 * kStatsBlocks + 1))) != cudaSuccess)
         return bail(e, "cudaMalloc(partials)");
@@ -682,6 +719,8 @@ rkl_status rkl_plan_destroy(rkl_plan* p)
         if (g.exec) cudaGraphExecDestroy(g.exec);
     for (int k = 0; k < 3; ++k) cudaFree(p->ybuf[k]);
     cudaFree(p->ybuf4);
+    cudaFree(p->padT);
+    cudaFree(p->padb);
     cudaFree(p->my0);
     if (p->s_in) cudaStreamSynchronize(p->s_in);
     if (p->s_out) cudaStreamSynchronize(p->s_out);

@@ -21,6 +21,7 @@ struct KGrid {
     R inv_4dx[3];        // 1/(4 dx_d)  (transverse gradient, Eq. qT)
     int64_t plane;       // n[0] * n[1]
     int64_t ncell;
+    int pitch;           // cells from one row to the next (row-padded arrays only; plane, ncell then count it)
 };
 
 // Conduction physics as the kernels see it (rho = 1, gamma = 2).

@@ -20,6 +20,7 @@ struct StageIO {
     const void* coef_tab;   // if non-null: coefficients at coef_tab[4 j .. 4 j + 3]
     int j;
     int mode;
+    bool padded;            // every array in the plan's row-padded layout
     bool chained;           // follows another stage launch of the same graph (launch_chained)
 };
 
@@ -130,6 +131,14 @@ cudaError_t launch_stage_xq(const LaunchCfg& c, const KGrid<float>& g, const KPh
 bool xg_stage_supported(const LaunchCfg& c, const KGrid<float>& g);
 cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
                             const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st);
+
+// The same kernel on row-padded arrays (g: pitch a multiple of four cells above
+// n[0], plane and ncell counting it; nx % 4 != 0), and the copies of T and b
+// into such arrays and of T back.
+cudaError_t launch_stage_xp(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
+                            const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st);
+cudaError_t launch_pack_rows(const KGrid<float>& g, const void* T, const void* b, void* pT, void* pb, cudaStream_t st);
+cudaError_t launch_unpack_rows(const KGrid<float>& g, const void* pT, void* T, cudaStream_t st);
 
 // Two-stage paired-cell FP32 3D kernel: stages j (io, coefficients at
 // io.coef_tab[4 j]) and j + 1 (written to Yj1) in one pass, 60 x 7 tiles of

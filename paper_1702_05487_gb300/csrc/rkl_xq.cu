@@ -184,6 +184,68 @@ cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPh
     return xq::launch_q_gen(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st, io.chained);
 }
 
+namespace xq {
+
+// Rows of nx cells (T, and the three components of b) into rows of `pitch`
+// cells, four at a time; blockIdx.y: array.  The padding is not read.
+__global__ void __launch_bounds__(256) pack_rows_kernel(const float* __restrict__ T, const float* __restrict__ b,
+                                                        float* __restrict__ pT, float* __restrict__ pb, unsigned chunks,
+                                                        int nx, int pitch, int64_t ncell, int64_t npad)
+{
+    const unsigned q = blockIdx.x * 256u + threadIdx.x, cpr = (unsigned)pitch / 4u;
+    if (q >= chunks) return;
+    const unsigned row = q / cpr, c = 4u * (q - row * cpr);
+    const float* s = (blockIdx.y == 0 ? T : b + (int64_t)(blockIdx.y - 1) * ncell) + (int64_t)row * nx + c;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int n = nx - (int)c;
+    v.x = s[0];
+    if (n > 1) v.y = s[1];
+    if (n > 2) v.z = s[2];
+    if (n > 3) v.w = s[3];
+    reinterpret_cast<float4*>(blockIdx.y == 0 ? pT : pb + (int64_t)(blockIdx.y - 1) * npad)[q] = v;
+}
+__global__ void __launch_bounds__(256) unpack_rows_kernel(const float* __restrict__ pT, float* __restrict__ T,
+                                                          unsigned chunks, int nx, int pitch)
+{
+    const unsigned q = blockIdx.x * 256u + threadIdx.x, cpr = (unsigned)pitch / 4u;
+    if (q >= chunks) return;
+    const unsigned row = q / cpr, c = 4u * (q - row * cpr);
+    const float4 v = reinterpret_cast<const float4*>(pT)[q];
+    float* d = T + (int64_t)row * nx + c;
+    const int n = nx - (int)c;
+    d[0] = v.x;
+    if (n > 1) d[1] = v.y;
+    if (n > 2) d[2] = v.z;
+    if (n > 3) d[3] = v.w;
+}
+
+}  // namespace xq
+
+cudaError_t launch_pack_rows(const KGrid<float>& g, const void* T, const void* b, void* pT, void* pb, cudaStream_t st)
+{
+    const int64_t chunks = g.ncell / 4, ncell = (int64_t)g.n[0] * g.n[1] * g.n[2];
+    xq::pack_rows_kernel<<<dim3((unsigned)((chunks + 255) / 256), 4), 256, 0, st>>>(
+        static_cast<const float*>(T), static_cast<const float*>(b), static_cast<float*>(pT), static_cast<float*>(pb),
+        (unsigned)chunks, g.n[0], g.pitch, ncell, g.ncell);
+    return cudaGetLastError();
+}
+cudaError_t launch_unpack_rows(const KGrid<float>& g, const void* pT, void* T, cudaStream_t st)
+{
+    const int64_t chunks = g.ncell / 4;
+    xq::unpack_rows_kernel<<<(unsigned)((chunks + 255) / 256), 256, 0, st>>>(
+        static_cast<const float*>(pT), static_cast<float*>(T), (unsigned)chunks, g.n[0], g.pitch);
+    return cudaGetLastError();
+}
+cudaError_t launch_stage_xp(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
+                            const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st)
+{
+    if (!xg_stage_supported(c, g) || g.pitch % 4 != 0) return cudaErrorNotSupported;
+    int nzc = nzchunk > 0 ? nzchunk : xq::auto_nzchunk_q(g, 64, xq::SmemQ<64>::TY);
+    nzc = std::max(nzc, (g.n[2] + 65534) / 65535);      // the grid's z limit
+    return (c.limiter ? xq::launch_q_pad_lim : xq::launch_q_pad)(c.spitzer != 0, c.saturate != 0, io.mode, g, p,
+                                                                 x2_args(io), coef, status, nzc, st, io.chained);
+}
+
 cudaError_t launch_ensemble_xq(bool spitzer, bool saturate, const x2::EnsProb* probs, const x2::EnsSeg* segs,
                                int nseg, int total, int* work, unsigned* done, unsigned* status, int* abort_flag,
                                long long spin_limit, int grid, cudaStream_t st)

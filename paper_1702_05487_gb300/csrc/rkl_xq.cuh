@@ -33,16 +33,18 @@
 // paired-cell kernel (rkl_x2_tile.cuh), so the two kernels write the same
 // bits.  Grids with fewer than 2^31 cells: periodic with nx % 4 == 0, or
 // (GEN builds) any width and either boundary, or (DIR builds) Dirichlet with
-// nx % 4 == 0, which keep the 16-byte chunks.  A GEN build copies rows in
+// nx % 4 == 0, which keep the 16-byte chunks, or (PAD builds) any other width
+// in arrays whose rows are padded to a multiple of four cells, which keep them
+// too.  A GEN build copies rows in
 // 4-byte pieces, one cell per lane, because 16-byte chunks of a row start
-// aligned in global memory only if nx % 4 == 0: a warp's copy of 32 cells is
-// then one or two 128-byte lines, so the shared-memory and L1 traffic stay
-// those of the 16-byte copies and the price is issue slots (33 copies a
-// thread and plane instead of 9).  Each lane's wrapped or clamped column and
-// row offsets are fixed per tile; Dirichlet ghosts of T are stored, not
-// copied.  201 x 150 x 99 stage: 138 us (one-cell tiled kernel) ->
-// 38 us.  Dirichlet 192 x 128 x 96, constant kappa: paired-cell 29
-// us, GEN 22, DIR 16.
+// aligned in global memory only if nx % 4 == 0; each lane's wrapped or clamped
+// column and row offsets are fixed per tile, Dirichlet ghosts of T are stored,
+// not copied.  33 copies a thread and plane instead of 9 throttle the memory
+// pipe (MIO stalls 1.6 cycles an issue against 0.2), so the single-stage entry
+// points take GEN, while super-steps take DIR or PAD.  201 x 150 x 99 stage:
+// one-cell tiled kernel 138 us, GEN 38, PAD 31 (and 20 us a super-step for the
+// copies).  Dirichlet 192 x 128 x 96, constant kappa: paired-cell 29 us, GEN
+// 22, DIR 16.
 #pragma once
 
 #include <algorithm>
@@ -164,12 +166,12 @@ __device__ __forceinline__ Pos tb_pos(const KGrid<float>& g, int t, int i0, int 
 }
 
 template <class SM>
-__device__ __forceinline__ Pos y_pos(const KGrid<float>& g, int t, int i0, int j0)
+__device__ __forceinline__ Pos y_pos(const KGrid<float>& g, int t, int i0, int j0, int rs)
 {
     constexpr int TX = SM::TX;
     const int row = t / (TX / 4), cc = (t % (TX / 4)) * 4;
     if (j0 + row >= g.n[1] || i0 + cc >= g.n[0]) return Pos{0u, ~0u};
-    return Pos{(unsigned)(j0 + row) * (unsigned)g.n[0] + (unsigned)(i0 + cc), (unsigned)((row * TX + cc) * 4)};
+    return Pos{(unsigned)(j0 + row) * (unsigned)rs + (unsigned)(i0 + cc), (unsigned)((row * TX + cc) * 4)};
 }
 
 __device__ __forceinline__ void cp4(unsigned d, const void* s)
@@ -226,7 +228,7 @@ __device__ __forceinline__ GenPos<SM> gen_pos(const KGrid<float>& g, int tid, in
 // and chunks past the edge are ghosts, flagged in the low bits of dst: T is
 // stored, and of a b chunk past the x edge only the cell beside the grid is
 // used, which repeats the edge cell (one 4-byte copy).
-enum : unsigned { PF_GHOST = 1u, PF_LEFT = 2u, PF_RIGHT = 4u, PF_ALL = 15u };
+enum : unsigned { PF_GHOST = 1u, PF_LEFT = 2u, PF_RIGHT = 4u, PF_PART = 8u, PF_ALL = 15u };
 template <class SM>
 __device__ __forceinline__ Pos dir_pos(const KGrid<float>& g, int t, int i0, int j0)
 {
@@ -239,7 +241,28 @@ __device__ __forceinline__ Pos dir_pos(const KGrid<float>& g, int t, int i0, int
     return Pos{(unsigned)clampi(gy, g.n[1]) * (unsigned)g.n[0] + (unsigned)sx, (unsigned)(SM::off(row, cc) * 4) | f};
 }
 
-enum { Q_PERIODIC = 0, Q_GEN = 1, Q_DIR = 2 };      // how a tile's bundles are copied
+// Copy positions of a PAD build (rows padded to a multiple of four cells, nx
+// % 4 != 0, either boundary): the chunks start aligned again.  The chunk left
+// of the grid brings its one used cell, the chunk that the row ends in comes
+// cell by cell with the cell beside the grid (wrapped or, Dirichlet, the edge
+// cell and a ghost T); chunks further out are not read.
+template <class SM>
+__device__ __forceinline__ Pos pad_pos(const KGrid<float>& g, int t, int i0, int j0)
+{
+    const int row = t / SM::CPR - 1, cc = (t % SM::CPR) * 4 - 4;
+    const int gx = i0 + cc, nx = g.n[0];
+    if (t >= SM::kPos || gx >= nx) return Pos{0u, ~0u};
+    int gy = j0 + row;
+    const bool ghost = g.bc == 1 && (gy < 0 || gy >= g.n[1]);
+    gy = g.bc == 1 ? clampi(gy, g.n[1]) : x2::pmod(gy, g.n[1]);
+    const int sx = gx < 0 ? (g.bc == 1 ? 0 : nx - 1) : gx;
+    return Pos{(unsigned)gy * (unsigned)g.pitch + (unsigned)sx,
+               (unsigned)(SM::off(row, cc) * 4) | (ghost ? PF_GHOST : 0u) | (gx < 0 ? PF_LEFT : 0u) |
+                   (gx + 3 >= nx ? PF_PART : 0u)};
+}
+
+// How a tile's bundles are copied.
+enum { Q_PERIODIC = 0, Q_GEN = 1, Q_DIR = 2, Q_PAD = 3 };
 
 template <bool SP, bool SAT, int MODE, int TXW, bool KP0 = false, bool LIM = false, int EDGE = Q_PERIODIC>
 __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, const KPhys<float>& p,
@@ -247,7 +270,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
                                        int z0, int nzc)
 {
     using Smem = SmemQ<TXW>;
-    constexpr bool GEN = EDGE == Q_GEN, DIR = EDGE == Q_DIR;
+    constexpr bool GEN = EDGE == Q_GEN, DIR = EDGE == Q_DIR, PAD = EDGE == Q_PAD;
     constexpr int TX = Smem::TX, TY = Smem::TY, LPR = Smem::LPR, SEGS = Smem::SEGS;
     constexpr int PLANE = Smem::PLANE;
     const int tid = threadIdx.x;
@@ -258,6 +281,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     const int ra = 2 * rp, rb = ra + 1;
     const int c = 2 * lx;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const int rs = PAD ? g.pitch : nx;          // cells from one row to the next
 
     if (MODE != 0 && a.coef_tab) {
         const float* t = a.coef_tab + 4 * a.j;
@@ -269,9 +293,12 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     if (GEN) {
         gp = gen_pos<Smem>(g, tid, i0, j0);
     } else {
-        p0 = DIR ? dir_pos<Smem>(g, tid, i0, j0) : tb_pos<Smem>(g, tid, i0, j0);
-        p1 = DIR ? dir_pos<Smem>(g, tid + NTHREADS, i0, j0) : tb_pos<Smem>(g, tid + NTHREADS, i0, j0);
-        if (MODE == 2) py = y_pos<Smem>(g, tid, i0, j0);
+        auto pos = [&](int t) {
+            return PAD ? pad_pos<Smem>(g, t, i0, j0) : (DIR ? dir_pos<Smem>(g, t, i0, j0) : tb_pos<Smem>(g, t, i0, j0));
+        };
+        p0 = pos(tid);
+        p1 = pos(tid + NTHREADS);
+        if (MODE == 2) py = y_pos<Smem>(g, tid, i0, j0, rs);
     }
     const float* bxp = a.b;
     const float* byp = a.b + g.ncell;
@@ -287,7 +314,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     // T and b of plane k, and (stages j >= 2) the Y bundle of plane k - 1
     auto load = [&](int k) {
         int kz = z0 + k;
-        const bool zg = (DIR || (GEN && g.bc == 1)) && (kz < 0 || kz >= nz);
+        const bool zg = (DIR || ((GEN || PAD) && g.bc == 1)) && (kz < 0 || kz >= nz);
         if (zg) kz = kz < 0 ? 0 : nz - 1;       // Dirichlet: ghosts, b of the nearest plane
         kz += kz < 0 ? nz : 0;                  // periodic: wrap the plane index
         kz -= kz >= nz ? nz : 0;
@@ -332,6 +359,29 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
         }
         auto copy = [&](const Pos& p) {
             const unsigned x = p.src + pt;
+            if (PAD && ((p.dst & PF_ALL) || zg)) {
+                const unsigned d = p.dst & ~PF_ALL;
+                const bool tg = zg || (p.dst & PF_GHOST);
+                auto one = [&](unsigned e, unsigned src, bool ghost) {
+                    if (ghost) st1(ts + d + e, g.bcv);
+                    else cp4(ts + d + e, a.Tin + src);
+                    cp4(bs + d + e, bxp + src);
+                    cp4(bs + PLANE * 4 + d + e, byp + src);
+                    cp4(bs + 2 * PLANE * 4 + d + e, bzp + src);
+                };
+                if (p.dst & PF_LEFT) one(12u, x, tg || g.bc == 1);
+                else if (p.dst & PF_PART) {
+                    const unsigned m = (unsigned)(nx & 3);          // cells of the row in its last chunk
+                    for (unsigned e = 0; e < m; ++e) one(4u * e, x + e, tg);
+                    one(4u * m, g.bc == 1 ? x + m - 1u : x + m - (unsigned)nx, tg || g.bc == 1);
+                } else {
+                    x2::st4(ts + d, g.bcv);
+                    cp16(bs + d, bxp + x);
+                    cp16(bs + PLANE * 4 + d, byp + x);
+                    cp16(bs + 2 * PLANE * 4 + d, bzp + x);
+                }
+                return;
+            }
             if (DIR && ((p.dst & PF_ALL) || zg)) {
                 const unsigned d = p.dst & ~PF_ALL;
                 if (zg || (p.dst & PF_GHOST)) x2::st4(ts + d, g.bcv);
@@ -353,7 +403,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
             cp16(bs + PLANE * 4 + p.dst, byp + x);
             cp16(bs + 2 * PLANE * 4 + p.dst, bzp + x);
         };
-        copy(p0);
+        if (!PAD || p0.dst != ~0u) copy(p0);
         if (p1.dst != ~0u) copy(p1);
         if (MODE == 2 && k >= 1 && py.dst != ~0u) {
             // plane k - 1 lies inside the chunk, so inside the grid
@@ -398,8 +448,8 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     float2 Tm0 = A.T0, Tm1 = A.T1, TmU = A.TU;
     float Tmr0 = A.r0, Tmr1 = A.r1;
 
-    const bool inx = i0 + c < nx;               // both cells or none, unless GEN: then perhaps the first alone
-    const bool in2 = !GEN || i0 + c + 1 < nx;
+    const bool inx = i0 + c < nx;               // both cells or none, unless GEN or PAD: then perhaps the first alone
+    const bool in2 = !(GEN || PAD) || i0 + c + 1 < nx;
     const bool vec = !GEN || (nx & 1) == 0;     // pairs are 8-byte aligned
     auto put = [&](float* o, float2 v) {
         if (vec) *reinterpret_cast<float2*>(o) = v;
@@ -411,7 +461,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
     // the check's operand: an odd width's last pair repeats its first cell
     auto seen = [&](float2 y) { return in2 ? y : bc2(y.x); };
     const bool in0 = inx && j0 + ra < ny, in1 = inx && j0 + rb < ny;
-    int64_t cbase = ((int64_t)z0 * ny + (j0 + ra)) * nx + (i0 + c);
+    int64_t cbase = ((int64_t)z0 * ny + (j0 + ra)) * rs + (i0 + c);
 
     // Pending between a plane and the next barrier: the divergence without
     // row 2w's lower y-face and without the left boundary face (lane 0),
@@ -452,7 +502,7 @@ __device__ __forceinline__ void tile_q(SmemQ<TXW>& sm, const KGrid<float>& g, co
             M1.x = fmaf(sm.FxLo[par][rb], -cmx.x, M1.x);
         }
         if (in0) emit(pcb, M0, Tm0, y00, yj0, my0);
-        if (in1) emit(pcb + nx, M1, Tm1, y01, yj1, my1);
+        if (in1) emit(pcb + rs, M1, Tm1, y01, yj1, my1);
     };
 
     // one plane: cur holds plane q, nxt receives plane q + 1
@@ -628,8 +678,8 @@ cudaError_t launch_q_lim(bool sp, bool sat, int mode, const KGrid<float>& g, con
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
                          cudaStream_t st, bool chained);
 // Builds for other grids, 64-column tiles, with the plain or (_lim) the
-// MC-limited gradients: GEN (rkl_xg.cu, rkl_xg_lim.cu) and DIR (rkl_xd.cu,
-// rkl_xd_lim.cu).
+// MC-limited gradients: GEN (rkl_xg.cu, rkl_xg_lim.cu), DIR (rkl_xd.cu,
+// rkl_xd_lim.cu) and PAD (rkl_xp.cu, rkl_xp_lim.cu).
 cudaError_t launch_q_gen(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
                          cudaStream_t st, bool chained);
@@ -640,6 +690,12 @@ cudaError_t launch_q_dir(bool sp, bool sat, int mode, const KGrid<float>& g, con
                          const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
                          cudaStream_t st, bool chained);
 cudaError_t launch_q_dir_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
+                             const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
+                             cudaStream_t st, bool chained);
+cudaError_t launch_q_pad(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
+                         const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
+                         cudaStream_t st, bool chained);
+cudaError_t launch_q_pad_lim(bool sp, bool sat, int mode, const KGrid<float>& g, const KPhys<float>& p,
                              const x2::FastArgs& a, const KCoef<float>& cf, unsigned* status, int nzchunk,
                              cudaStream_t st, bool chained);
 
