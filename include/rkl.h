@@ -471,7 +471,7 @@ rkl_status rkl_sur_features(rkl_surrogate *sur, const void *T, const void *b, do
  * warp-level mma.sync kernels, 1 the tcgen05 kernels (M = 128-voxel blocks
  * of one plane, accumulators in tensor memory; needs W % 8 == 0 and
  * H % 16 == 0, else RKL_ERR_UNSUPPORTED).  The default is 1 where the
- * patch allows it.  Weight gradients use the warp-level kernel either way.
+ * patch allows it.  Weight gradients run on tcgen05 either way.
  */
 rkl_status rkl_sur_set_backend(rkl_surrogate *sur, int backend);
 /*
@@ -518,7 +518,7 @@ rkl_status rkl_sur_train_step(rkl_surrogate *sur, double head_scale, const void 
  *                  sum_v dz[v][co] x[v + o][ci], db[co] = sum_v dz[v][co],
  *                  summed in a fixed order (the same result every run).
  * The forward and backward-data passes use the backend of
- * rkl_sur_set_backend; the weight gradient is the warp-level kernel.
+ * rkl_sur_set_backend; the weight gradient is a tcgen05 kernel.
  * (cin, cout) of a layer: rkl_sur_layer_shape.
  */
 rkl_status rkl_sur_layer_forward(rkl_surrogate *sur, int layer, const void *in, void *out);

@@ -1,6 +1,7 @@
 // Kernels of the learned surrogate: periodic 3x3x3 convolutions as implicit
-// GEMMs on BF16 tensor cores (mma.sync m16n8k16, FP32 accumulation), their
-// backward passes, the flux-form head, the MSE loss and Adam.
+// GEMMs on BF16 tensor cores (mma.sync m16n8k16, FP32 accumulation), forward
+// and backward-data (the weight gradient is in rkl_wgrad_tc.cu), the flux-form
+// head, the MSE loss and Adam.
 //
 // Layouts (voxel v = (z * H + y) * W + x of a periodic D x H x W patch):
 //   activations  bf16 [V][C]            (channels last, C = 16 or 32)

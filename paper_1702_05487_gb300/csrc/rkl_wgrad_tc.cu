@@ -490,7 +490,7 @@ cudaError_t conv_wgrad_tc(int cin, int cout, const void* dz, const void* x, floa
                           int H, int W, unsigned* status, cudaStream_t st)
 {
     if (H % BY || W % BX || D % 4) return cudaErrorInvalidValue;
-    if ((int64_t)H * W * 32 >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;      // 32-bit in-plane offsets
+    if ((int64_t)H * W * 32 > ((int64_t)1 << 31)) return cudaErrorInvalidValue;       // 31-bit in-plane offsets
     if (cin == 16 && cout == 32) return wgrad_tc_t<16, 32>(dz, x, dW, db, part, D, H, W, status, st);
     if (cin == 32 && cout == 32) return wgrad_tc_t<32, 32>(dz, x, dW, db, part, D, H, W, status, st);
     if (cin == 32 && cout == 16) return wgrad_tc_t<32, 16>(dz, x, dW, db, part, D, H, W, status, st);
