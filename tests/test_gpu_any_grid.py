@@ -81,3 +81,19 @@ def test_bad_cells_are_reported(rk, dtype, shape):  # noqa: F811
     neg.view(-1)[-1] = -1e-3
     plan.super_step_s(1e-9 * dt, 2, neg, torch.zeros_like(bd))
     assert plan.check() == 4                     # RKL_ERR_NONPOSITIVE_T
+
+
+def test_new_ensemble_schedule_same_bits(rk):  # noqa: F811
+    """The schedule an ensemble starts with (row-pair tiles, a tile length
+    from its sizes) advances it to the bits of the paired-cell schedule."""
+    import torch
+    from test_gpu_ensemble import _build, _periodic_specs
+    got = []
+    for sched in (None, (1, 32)):
+        ens, T_all, b_all, _, _, dts = _build(rk, _periodic_specs())
+        if sched:
+            ens.set_schedule(*sched)
+        ens.super_step(dts, T_all, b_all)
+        assert ens.check() == 0
+        got.append(T_all.clone())
+    assert torch.equal(got[0], got[1])
