@@ -29,7 +29,7 @@
 // up dz for the bias.  Every wait is bounded and reports ST_TIMEOUT.
 //
 // 32 -> 32 channels: 128^3 121 us with the slices' sum (the warp-level
-// mma.sync kernel before it: about 320), 96^3 62 us (206).  The MMAs alone
+// mma.sync kernel before it: about 360), 96^3 64 us (about 180).  The MMAs alone
 // (three of 128 x 96 x 16 per 16 voxels, a quarter of M idle) take 97 us of
 // the 121, the copies alone 113; with one issuing thread it was 157 us, with
 // a window of three steps 222 us (each step then waited for the one before).
