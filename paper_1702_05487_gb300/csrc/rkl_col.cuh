@@ -50,17 +50,16 @@ struct Args {
     int mode;
 };
 
-// Square root: FP32 as everywhere; FP64 as the reciprocal square root
-// estimate of the PTX ISA refined by one third-order (Householder) step,
-// sqrt(x) = t (1 + e / 2 + 3 e^2 / 8) with t = x r, e = 1 - t r: with an
-// estimate good to 2^-19 the remainder 5 e^3 / 16 is below 2^-55, five FP64
-// operations.  Anything but positive normal numbers takes sqrt().
-template <typename R>
-__device__ __forceinline__ R root(R x);
-template <>
-__device__ __forceinline__ float root<float>(float x) { return dsqrt<float>(x); }
-template <>
-__device__ __forceinline__ double root<double>(double x)
+// Square root of an FP64 number: the reciprocal square root estimate r of the
+// PTX ISA refined by one third-order (Householder) step, sqrt(x) = t (1 + e / 2
+// + 3 e^2 / 8) with t = x r, e = 1 - t r, five FP64 operations.  The rounding of
+// t is part of e; with |e| <= 2^-19 the remainder 5 e^3 / 16 is below 2^-58 of the
+// root: within 0.52 ulp.  Of 25 million roots 0.06% were not the rounded one, by
+// at most 0.515 ulp; the error of M against 80-bit arithmetic is that with sqrt()
+// and below the generic kernel's (rms 2.2e-16 against 2.6e-16 of M's rms).  With
+// sqrt() a Spitzer stage takes 5% longer and a saturated one 10%.  Anything but
+// positive normal numbers takes sqrt().
+__device__ __forceinline__ double root(double x)
 {
     if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fe00000u) return sqrt(x);
     double r;
@@ -115,7 +114,7 @@ __device__ __forceinline__ R face(R TL, R TR, R gn, R g1, R g2, R Bn, R B1, R B2
     R X = Bn * bdg;
     const bool perp = k.kp4 != R(0);
     if (perp) X += k.kp4 * gn;
-    if (!SAT) return SP ? (Ts * Ts) * root<R>(Ts) * X : X;
+    if (!SAT) return SP ? (Ts * Ts) * root(Ts) * X : X;
     R Y1 = B1 * bdg;
     R Y2 = ND == 3 ? B2 * bdg : R(0);
     if (perp) {
@@ -125,16 +124,16 @@ __device__ __forceinline__ R face(R TL, R TR, R gn, R g1, R g2, R Bn, R B1, R B2
     R V2 = X * X + Y1 * Y1;
     if (ND == 3) V2 += Y2 * Y2;
     if (!p.upwind) {
-        const R sTs = root<R>(Ts), Vm = root<R>(V2);
+        const R sTs = root(Ts), Vm = root(V2);
         if (SP) return ddiv<R>((Ts * Ts) * sTs * X, k.sat * (Ts * Vm) + R(1));
         const R T15 = Ts * sTs;
         return ddiv<R>(T15 * X, k.sat * Vm + T15);
     }
-    const R nk = SP ? k.nk * (Ts * Ts) * root<R>(Ts) : k.nk;
+    const R nk = SP ? k.nk * (Ts * Ts) * root(Ts) : k.nk;
     const R Fn = nk * X;
     const R Tq = Fn >= R(0) ? TL : TR;
-    const R q = p.q0 * Tq * root<R>(Tq);
-    return ddiv<R>(q, q + fabs(nk) * root<R>(V2)) * Fn;
+    const R q = p.q0 * Tq * root(Tq);
+    return ddiv<R>(q, q + fabs(nk) * root(V2)) * Fn;
 }
 
 // A cell's transverse slope along one axis: the centred difference and, with
