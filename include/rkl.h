@@ -489,8 +489,17 @@ rkl_status rkl_sur_features_flux(rkl_surrogate *sur, rkl_plan *plan, const void 
  * default): rkl_sur_features */
 rkl_status rkl_sur_set_flux_features(rkl_surrogate *sur, double c);
 /* waits for the stream; RKL_ERR_TIMEOUT if a tcgen05 kernel's bounded wait
- * gave up since the last check (the word is then cleared) */
+ * gave up since the last check (the word is then cleared).  Until then
+ * rkl_sur_backward, rkl_sur_get_grads, rkl_sur_adam and rkl_sur_train_step
+ * return RKL_ERR_TIMEOUT too, and no parameter changes: gradients behind
+ * such a wait are unfinished sums. */
 rkl_status rkl_sur_check(rkl_surrogate *sur);
+/*
+ * Failure-detection self-test: one bounded wait of the gradient kernel, with a
+ * short limit, on a barrier that nothing arrives at.  It must give up; the
+ * calls above then report RKL_ERR_TIMEOUT.
+ */
+rkl_status rkl_sur_selftest_timeout(rkl_surrogate *sur);
 /* forward pass; the increment dT goes to dT_out (device floats) if not NULL */
 rkl_status rkl_sur_forward(rkl_surrogate *sur, double head_scale, void *dT_out);
 /* MSE loss 0.5 mean((dT - target)^2) of the last forward and all gradients */

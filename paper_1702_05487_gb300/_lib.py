@@ -103,6 +103,7 @@ SIGNATURES = {
     "rkl_sur_features": (ctypes.c_int, [_vp, _vp, _vp, ctypes.c_double, ctypes.c_int, ctypes.c_double]),
     "rkl_sur_set_backend": (ctypes.c_int, [_vp, ctypes.c_int]),
     "rkl_sur_check": (ctypes.c_int, [_vp]),
+    "rkl_sur_selftest_timeout": (ctypes.c_int, [_vp]),
     "rkl_sur_forward": (ctypes.c_int, [_vp, ctypes.c_double, _vp]),
     "rkl_sur_backward": (ctypes.c_int, [_vp, _vp, _dp]),
     "rkl_sur_adam": (ctypes.c_int, [_vp, ctypes.c_double, ctypes.c_double, ctypes.c_double, ctypes.c_double]),
@@ -459,6 +460,11 @@ def rkl_sur_set_backend(sur, backend: int):
 
 def rkl_sur_check(sur):
     _scheck(load().rkl_sur_check(sur), sur)
+
+
+def rkl_sur_selftest_timeout(sur):
+    """Lets one bounded wait run out: the gradient calls then raise until rkl_sur_check has."""
+    _scheck(load().rkl_sur_selftest_timeout(sur), sur)
 
 
 def rkl_sur_forward(sur, head_scale, dT_out=None):

@@ -30,6 +30,9 @@ size_t wgrad_workspace_floats();
 cudaError_t conv_wgrad_tc(int cin, int cout, const void* dz, const void* x, float* dW, float* db, float* part, int D,
                           int H, int W, unsigned* status, cudaStream_t st);
 
+// Lets a bounded wait of that kernel run out (sets ST_TIMEOUT in *status).
+cudaError_t wait_selftest(unsigned* status, cudaStream_t st);
+
 cudaError_t features(const float* T, const float* b, int64_t V, float kappa0, int spitzer, float ratio, const float* F,
                      float fscale, void* X, cudaStream_t st);
 cudaError_t head_div(const float* G, int D, int H, int W, float tau, const float inv_dx[3], float* dT,

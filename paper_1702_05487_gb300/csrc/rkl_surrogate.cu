@@ -116,6 +116,8 @@ struct rkl_surrogate {
     float* Mp = nullptr;
     int backend = 0;               // 0: warp-level mma.sync convolutions, 1: tcgen05
     unsigned* d_tcst = nullptr;    // status word of the tcgen05 kernels' bounded waits
+    unsigned* h_tcst = nullptr;    // as last read (pinned, behind h_part); kept until rkl_sur_check
+    bool tc_unread = false;        // a layer's weight gradient was launched since
     double* d_part = nullptr;
     double* h_part = nullptr;      // pinned
     bool forward_done = false;
@@ -137,6 +139,15 @@ rkl_status sfail(rkl_surrogate* s, rkl_status st, const std::string& m)
         cudaError_t c_ = (call);                                                                          \
         if (c_ != cudaSuccess) return sfail((s), RKL_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(c_)); \
     } while (0)
+
+// Whether the gradients may be used, from the status word as last read: sums
+// behind a wait that gave up are unfinished.
+rkl_status grads_ok(rkl_surrogate* s)
+{
+    if (*s->h_tcst & ST_TIMEOUT)
+        return sfail(s, RKL_ERR_TIMEOUT, "a bounded wait of a tensor-core kernel gave up: the gradients are not valid");
+    return RKL_OK;
+}
 
 size_t wcount(int l) { return (size_t)27 * kCout[l] * kCin[l]; }
 
@@ -185,7 +196,11 @@ rkl_status backward_impl(rkl_surrogate* s, const float* target, double* loss)
             cur = 1 - cur;
         }
     }
+    SUR_CK(s, cudaMemcpyAsync(s->h_tcst, s->d_tcst, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
     SUR_CK(s, cudaStreamSynchronize(s->stream));
+    s->tc_unread = false;
+    rkl_status st = grads_ok(s);
+    if (st != RKL_OK) return st;
     double acc = 0.0;
     for (int k = 0; k < kPartials; ++k) acc += s->h_part[k];
     if (loss) *loss = 0.5 * acc / (double)s->V;
@@ -267,7 +282,10 @@ rkl_status rkl_sur_create(int D, int H, int W, const double* dx, void* cuda_stre
         return bail(c, "gradient partials");
     if ((c = cudaMalloc(&s->d_tcst, sizeof(unsigned))) != cudaSuccess) return bail(c, "status");
     if ((c = cudaMemsetAsync(s->d_tcst, 0, sizeof(unsigned), s->stream)) != cudaSuccess) return bail(c, "status");
-    if ((c = cudaMallocHost(&s->h_part, sizeof(double) * 2 * kPartials)) != cudaSuccess) return bail(c, "partials");
+    if ((c = cudaMallocHost(&s->h_part, sizeof(double) * (2 * kPartials + 1))) != cudaSuccess)
+        return bail(c, "partials");
+    s->h_tcst = reinterpret_cast<unsigned*>(s->h_part + 2 * kPartials);
+    *s->h_tcst = 0u;
     if ((c = cudaStreamSynchronize(s->stream)) != cudaSuccess) return bail(c, "sync");
     for (int l = 0; l < kLayers; ++l)
         if (pack_impl(s, l) != RKL_OK) return bail(cudaGetLastError(), "pack");
@@ -324,8 +342,11 @@ rkl_status rkl_sur_get_grads(rkl_surrogate* s, int layer, float* gw_host, float*
     if (!s || layer < 0 || layer >= kLayers || !gw_host || !gb_host) return RKL_ERR_INVALID_ARG;
     SUR_CK(s, cudaMemcpyAsync(gw_host, s->gw[layer], sizeof(float) * wcount(layer), cudaMemcpyDeviceToHost, s->stream));
     SUR_CK(s, cudaMemcpyAsync(gb_host, s->gb[layer], sizeof(float) * kCout[layer], cudaMemcpyDeviceToHost, s->stream));
+    if (s->tc_unread)
+        SUR_CK(s, cudaMemcpyAsync(s->h_tcst, s->d_tcst, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
     SUR_CK(s, cudaStreamSynchronize(s->stream));
-    return RKL_OK;
+    s->tc_unread = false;
+    return grads_ok(s);
 }
 
 rkl_status rkl_sur_features(rkl_surrogate* s, const void* T, const void* b, double kappa0, int spitzer, double ratio)
@@ -386,11 +407,21 @@ rkl_status rkl_sur_set_backend(rkl_surrogate* s, int backend)
 rkl_status rkl_sur_check(rkl_surrogate* s)
 {
     if (!s) return RKL_ERR_INVALID_ARG;
-    unsigned w = 0;
-    SUR_CK(s, cudaMemcpyAsync(&w, s->d_tcst, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
+    SUR_CK(s, cudaMemcpyAsync(s->h_tcst, s->d_tcst, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
     SUR_CK(s, cudaStreamSynchronize(s->stream));
     SUR_CK(s, cudaMemsetAsync(s->d_tcst, 0, sizeof(unsigned), s->stream));
+    const unsigned w = *s->h_tcst;
+    *s->h_tcst = 0u;
+    s->tc_unread = false;
     if (w & ST_TIMEOUT) return sfail(s, RKL_ERR_TIMEOUT, "a bounded wait of a tensor-core convolution gave up");
+    return RKL_OK;
+}
+
+rkl_status rkl_sur_selftest_timeout(rkl_surrogate* s)
+{
+    if (!s) return RKL_ERR_INVALID_ARG;
+    SUR_CK(s, conv::wait_selftest(s->d_tcst, s->stream));
+    s->tc_unread = true;
     return RKL_OK;
 }
 
@@ -413,6 +444,13 @@ rkl_status rkl_sur_backward(rkl_surrogate* s, const void* target, double* loss)
 rkl_status rkl_sur_adam(rkl_surrogate* s, double lr, double beta1, double beta2, double eps)
 {
     if (!s || !(lr > 0.0)) return RKL_ERR_INVALID_ARG;
+    if (s->tc_unread) {
+        SUR_CK(s, cudaMemcpyAsync(s->h_tcst, s->d_tcst, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
+        SUR_CK(s, cudaStreamSynchronize(s->stream));
+        s->tc_unread = false;
+    }
+    rkl_status ok = grads_ok(s);
+    if (ok != RKL_OK) return ok;
     s->adam_t += 1;
     for (int l = 0; l < kLayers; ++l) {
         SUR_CK(s, conv::adam(s->w[l], s->gw[l], s->mw[l], s->vw[l], (int)wcount(l), (float)lr, (float)beta1,
@@ -455,6 +493,7 @@ rkl_status rkl_sur_layer_weight_grad(rkl_surrogate* s, int layer, const void* dz
     if (!s || layer < 0 || layer >= kLayers || !dz || !x) return RKL_ERR_INVALID_ARG;
     SUR_CK(s, conv::conv_wgrad_tc(kCin[layer], kCout[layer], dz, x, s->gw[layer], s->gb[layer], s->gpart, s->D,
                                   s->H, s->W, s->d_tcst, s->stream));
+    s->tc_unread = true;
     return RKL_OK;
 }
 

@@ -119,6 +119,13 @@ __device__ __forceinline__ void tmem_ld16w(unsigned taddr, float* v)
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+// Bounded wait; false if it gave up.
+__device__ __forceinline__ bool wait_w(unsigned long long& bar, unsigned parity, int limit = 1 << 24)
+{
+    for (int it = 0; it < limit; ++it)
+        if (mbar_try_wait(smem_u32(&bar), parity)) return true;
+    return false;
+}
 __device__ __forceinline__ int wrapw(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
 // The CTA's run of (column, plane) units as segments of one column each.
@@ -172,12 +179,7 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ dz, const __nv_bfloat16* __res
     const unsigned xbase = smem_u32(&sm.X[0][0]), zbase = smem_u32(&sm.Z[0]);
     // bounded waits; a thread whose wait gave up skips its later ones
     bool ok = true;
-    auto wait = [&](unsigned long long& bar, unsigned parity) {
-        if (!ok) return;
-        for (int it = 0; it < (1 << 24); ++it)
-            if (mbar_try_wait(smem_u32(&bar), parity)) return;
-        ok = false;
-    };
+    auto wait = [&](unsigned long long& bar, unsigned parity) { ok = ok && wait_w(bar, parity); };
 
     Seg sg;
     int u = ubeg;
@@ -313,7 +315,8 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ dz, const __nv_bfloat16* __res
     // offsets +1, 0, -1; warps 4 .. 7 reach the lane quarters 0 .. 3
     __syncwarp();
     if (warp >= 4 && warp < 8) {
-        wait(sm.done, 0u);
+        // also after a wait that gave up: TMEM is given back only once the MMAs have ended
+        ok = wait_w(sm.done, 0u) && ok;
         __syncwarp();
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const int m = (warp & 3) * 32 + lane, r = m / COUT, co = m % COUT;
@@ -342,6 +345,14 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ dz, const __nv_bfloat16* __res
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tbase), "r"(TMEM_ALL) : "memory");
     }
     if (!ok && status) atomicOr(status, ST_TIMEOUT);
+}
+
+// One wait of the kernel above, short, on a barrier that nothing arrives at.
+__global__ void wait_selftest_kernel(unsigned* status)
+{
+    __shared__ unsigned long long bar;
+    mbar_init(smem_u32(&bar), 1u);
+    if (!wait_w(bar, 0u, 64)) atomicOr(status, ST_TIMEOUT);
 }
 
 // dW[i] = sum of the slices part[b][i] in a fixed order (eight strided runs,
@@ -485,6 +496,12 @@ cudaError_t wgrad_tc_t(const void* dz, const void* x, float* dW, float* db, floa
 }
 
 }  // namespace
+
+cudaError_t wait_selftest(unsigned* status, cudaStream_t st)
+{
+    wait_selftest_kernel<<<1, 1, 0, st>>>(status);
+    return cudaGetLastError();
+}
 
 cudaError_t conv_wgrad_tc(int cin, int cout, const void* dz, const void* x, float* dW, float* db, float* part, int D,
                           int H, int W, unsigned* status, cudaStream_t st)
