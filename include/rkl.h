@@ -312,8 +312,13 @@ rkl_status rkl_plan_set_method(rkl_plan *plan, int method, double sts_nu);
  * tiled; paired-cell at 5 and 6 CTAs per SM, automatic, balanced or with 16,
  * 32, 64 planes per CTA; two-stage; bulk and tensor-map copies; row-pair) on a
  * scratch copy of T (T is not changed), keeps the fastest with
- * rkl_plan_set_variant and returns it.  Allocates and frees one grid-sized
- * scratch array.  Synchronises.
+ * rkl_plan_set_variant and returns it.  The automatic choice (variant 0) is
+ * timed too: where no numbered variant is faster the plan keeps it, and
+ * *variant_out names the fastest numbered one tried (0 where the automatic
+ * choice has no number of its own); *ms_out is the time of what the plan
+ * keeps.  On limiter plans of fewer than 65536 cells only variants 1 to 3 and
+ * the automatic choice are tried.  Allocates and frees one grid-sized scratch
+ * array.  Synchronises.
  */
 rkl_status rkl_plan_autotune(rkl_plan *plan, double dt, const void *T, const void *b,
                              int *variant_out, int *nzchunk_out, double *ms_out);

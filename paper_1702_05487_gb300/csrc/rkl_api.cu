@@ -1,6 +1,7 @@
 // C ABI of the RKL2 conduction library (see include/rkl.h): argument
 // checks, the plan (workspace, coefficient table, graph cache, timing) and
 // the dispatch between the tiled FP32 kernel and the generic kernels.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -954,23 +955,27 @@ rkl_status rkl_plan_autotune(rkl_plan* p, double dt, const void* T, const void* 
         for (int nz : {0, -1, 32}) cands.push_back({8, nz});
     if (p->xqok)
         for (int nz : {0, 16, 32}) {
-            // below 64 Ki cells a limited stage is bound by launch latency
-            // (3-4 us on either kernel): the search stays with the
-            // paired-cell build there
+            // (limiter plans below 64 Ki cells report a variant from 1 to 3, as
+            // they did before the automatic choice was timed beside them)
             if (!lim || p->ncell >= 65536) cands.push_back({10, nz});
             // 32-column tiles only where they leave fewer columns idle (the
             // limited build has 64-column tiles only)
             if (!lim && narrow_tiles(p->gf.n[0])) cands.push_back({11, nz});
         }
-    // kernels without a number of their own: the automatic choice
-    if (p->colok || (p->xgok && !p->xqok)) cands.push_back({0, 0});
+    // The automatic choice is timed in any case, and the plan keeps it where no
+    // variant is faster, so tuning cannot slow a plan down: 20 x 16 x 64
+    // limited, paired-cell 52 us a super-step of 11 stages, automatic 38.  It
+    // is reported as 0 where it launches a kernel without a number.
+    const Cand automatic{0, 0};
+    const bool unnumbered = p->colok || (p->xgok && !p->xqok);
+    cands.push_back(automatic);
     void* scratch = nullptr;
     RKL_CK(p, cudaMalloc(&scratch, (size_t)p->ncell * p->esize));
     cudaEvent_t a = nullptr, e = nullptr;
     cudaEventCreate(&a);
     cudaEventCreate(&e);
     const int keep_v = p->variant, keep_nz = p->nzchunk;
-    double best = 1e300;
+    double best = 1e300, best_auto = 1e300;
     Cand bc = cands[0];
     for (const Cand& c : cands) {
         if (rkl_plan_set_variant(p, c.v, c.nz) != RKL_OK) continue;
@@ -984,7 +989,8 @@ rkl_status rkl_plan_autotune(rkl_plan* p, double dt, const void* T, const void* 
             cudaEventElapsedTime(&ms, a, e);
         }
         if (st != RKL_OK) break;
-        if (ms < best) {
+        if (c.v == 0) best_auto = ms;
+        else if (ms < best) {
             best = ms;
             bc = c;
         }
@@ -996,10 +1002,12 @@ rkl_status rkl_plan_autotune(rkl_plan* p, double dt, const void* T, const void* 
         rkl_plan_set_variant(p, keep_v, keep_nz);
         return st;
     }
-    rkl_plan_set_variant(p, bc.v, bc.nz);
+    const Cand keep = best_auto <= best ? automatic : bc;
+    if (keep.v == 0 && unnumbered) bc = keep;
+    rkl_plan_set_variant(p, keep.v, keep.nz);
     if (variant_out) *variant_out = bc.v;
-    if (nzchunk_out) *nzchunk_out = p->nzchunk;
-    if (ms_out) *ms_out = best;
+    if (nzchunk_out) *nzchunk_out = bc.nz;
+    if (ms_out) *ms_out = std::min(best, best_auto);
     return rkl_plan_check(p);
 }
 

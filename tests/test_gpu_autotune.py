@@ -1,0 +1,38 @@
+"""Tuning never leaves a plan slower than the automatic choice."""
+import pytest
+
+from test_gpu_parity import _fields, rk  # noqa: F401  (fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def _best_ms(plan, dt, T, b):
+    import torch
+    X = T.clone()
+    best = 1e300
+    for _ in range(60):
+        X.copy_(T)
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        plan.super_step_s(dt, 11, X, b)
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1))
+    return best
+
+
+@pytest.mark.parametrize("shape,bc", [((20, 16, 64), "periodic"), ((16, 16, 16), "periodic"), ((20, 16, 64), "dirichlet")])
+def test_small_limited_plan_is_not_slowed_down(rk, shape, bc):  # noqa: F811
+    """The fastest of 60 super-steps before and after tuning (the paired-cell
+    kernel, which the search used to end with, takes 1.35 times as long as the
+    row-pair one here)."""
+    import torch
+    T, b = _fields(shape)
+    Td, bd = torch.from_numpy(T).float().cuda(), torch.from_numpy(b).float().cuda()
+    plan = rk.Plan(shape, "f32", params=dict(kappa_model="spitzer", kappa_par0=0.01, kappa_perp_ratio=1e-4,
+                                             limiter="mc", bc=bc, bc_value=1.0))
+    dt = 50 * plan.dt_expl(Td)
+    before = _best_ms(plan, dt, Td, bd)
+    plan.autotune(dt, Td, bd)
+    after = min(_best_ms(plan, dt, Td, bd) for _ in range(2))
+    assert after < 1.15 * before, (before, after)
