@@ -158,8 +158,8 @@ rkl_status rkl_coeffs_method(int method, int s, double sts_nu, double *mu, doubl
  * passed as void*; NULL is the legacy default stream).  The plan allocates
  * its own device workspace: three stage buffers, M(Y_0), reduction scratch
  * (4 grid arrays plus a few KB; FP32 3D plans whose width is not a multiple of
- * four also hold copies of T and b with padded rows, where memory allows) and
- * caches one CUDA graph per distinct
+ * four allocate copies of T and b with padded rows, 4 more, at their first
+ * super-step of four or more stages, where memory allows) and caches one CUDA graph per distinct
  * (s, T, b) triple used by rkl_super_step.  The device current at creation
  * is used for every later call.  Writes *out; destroy with
  * rkl_plan_destroy.

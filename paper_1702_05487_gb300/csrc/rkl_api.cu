@@ -56,8 +56,8 @@ struct rkl_plan {
     bool xqok = false;                 // row-pair kernel applies to the grid
     bool xgok = false;                 // row-pair kernel for any width and boundary applies
     // FP32 3D widths that are not a multiple of four: super-steps run on
-    // row-padded arrays (the plan's buffers and copies of T and b), whose rows
-    // start 16-byte aligned
+    // row-padded arrays (the plan's buffers and copies of T and b, allocated on
+    // use), whose rows start 16-byte aligned
     bool padok = false;
     KGrid<float> gpad{};
     void* padT = nullptr;
@@ -267,14 +267,30 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
     return RKL_OK;
 }
 
+// Whether s stages run on row-padded copies.  201 x 150 x 99: the copies cost 20
+// us, a stage on padded rows takes 31 us, on the caller's 38 us, so they pay from
+// four stages on.
+bool wants_padding(const rkl_plan* p, int s) { return p->padok && p->variant == 0 && s >= 4; }
+
+// The row-padded copies, before the first super-step that wants them: plans that
+// only call single stages or short super-steps hold four grid arrays, not eight.
+void allocate_padding(rkl_plan* p)
+{
+    const size_t bytes = (size_t)p->gpad.ncell * p->esize;
+    if (cudaMalloc(&p->padT, bytes) == cudaSuccess && cudaMalloc(&p->padb, 3 * bytes) == cudaSuccess) return;
+    // no room: the stages read the caller's rows
+    cudaGetLastError();
+    cudaFree(p->padT);
+    p->padT = nullptr;
+    p->padok = false;
+}
+
 // Enqueue the s stages of one super-step reading coefficients from the
 // plan's device table (stage j at d_coef[4 j]).  Y0 = T; the last stage
 // writes T (each cell reads its own Y0 before overwriting it).
 rkl_status enqueue_stages(rkl_plan* p, int s, void* Tuser, const void* buser, bool with_events, cudaStream_t cs)
 {
-    // 201 x 150 x 99: the copies cost 20 us, a stage on padded rows takes 31 us,
-    // on the caller's 38 us, so they pay from four stages on
-    const bool padded = p->padok && p->variant == 0 && s >= 4;
+    const bool padded = wants_padding(p, s) && p->padT;
     void* T = padded ? p->padT : Tuser;
     const void* b = padded ? p->padb : buser;
     if (padded) RKL_CK(p, launch_pack_rows(p->gpad, Tuser, buser, p->padT, p->padb, cs));
@@ -294,8 +310,7 @@ rkl_status enqueue_stages(rkl_plan* p, int s, void* Tuser, const void* buser, bo
     rkl_status st = launch_stage(p, io, 0, 0, 0, 0, cs);
     if (st != RKL_OK) return st;
     if (s == 1) {                      // single forward-Euler stage (RKL1, AAG-STS)
-        if (padded) RKL_CK(p, launch_unpack_rows(p->gpad, p->ybuf[0], Tuser, cs));
-        else RKL_CK(p, cudaMemcpyAsync(T, p->ybuf[0], (size_t)p->ncell * p->esize, cudaMemcpyDeviceToDevice, cs));
+        RKL_CK(p, cudaMemcpyAsync(T, p->ybuf[0], (size_t)p->ncell * p->esize, cudaMemcpyDeviceToDevice, cs));
         return RKL_OK;
     }
     if (with_events) RKL_CK(p, cudaEventRecordWithFlags(p->ev_a, cs, cudaEventRecordExternal));
@@ -488,6 +503,7 @@ double dt_expl_from_max(const rkl_plan* p, double Tmax)
 
 rkl_status run_super_step(rkl_plan* p, double dt, int s, void* T, const void* b, double* eb, double* ea)
 {
+    if (wants_padding(p, s) && !p->padT) allocate_padding(p);
     rkl_status st = upload_coeffs(p, s, dt);
     if (st != RKL_OK) return st;
     cudaGraphExec_t exec = nullptr;
@@ -680,13 +696,6 @@ rkl_status rkl_plan_create(const rkl_grid* grid, const rkl_phys* phys, void* cud
     for (int k = 0; k < 3; ++k)
         if ((e = cudaMalloc(&p->ybuf[k], bytes)) != cudaSuccess) return bail(e, "cudaMalloc(stage buffer)");
     if ((e = cudaMalloc(&p->my0, bytes)) != cudaSuccess) return bail(e, "cudaMalloc(MY0)");
-    if (p->padok && (cudaMalloc(&p->padT, bytes) != cudaSuccess || cudaMalloc(&p->padb, 3 * bytes) != cudaSuccess)) {
-        // no room for the copies: the stages read the caller's rows
-        cudaGetLastError();
-        cudaFree(p->padT);
-        p->padT = nullptr;
-        p->padok = false;
-    }
     // partials of the statistics pass, then its block ticket counter (zeroed)
     if ((e = cudaMalloc(&p->d_partials, sizeof(double) * (3 * kStatsBlocks + 1))) != cudaSuccess)
         return bail(e, "cudaMalloc(partials)");
