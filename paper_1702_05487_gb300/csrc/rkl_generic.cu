@@ -1,8 +1,10 @@
 // Generic RKL2 conduction kernels: one thread per cell, any dtype (float /
-// double), 1-3 active axes, periodic or Dirichlet boundaries.  These serve
-// the FP64 and low-dimensional configurations and every case the tiled FP32
-// kernel does not cover; each cell evaluates the fluxes on all of its faces
-// straight from global memory (L1/L2 absorb the neighbour re-reads).
+// double), 1-3 active axes, periodic or Dirichlet boundaries.  The stage
+// kernel serves 1D grids, 2D FP32 grids with a finite limiter floor and what
+// the tiled and column-march kernels do not cover; each cell evaluates the
+// fluxes on all of its faces straight from global memory (L1/L2 absorb the
+// neighbour re-reads).  The face fluxes, the advection step and the statistics
+// of every grid are here too.
 #include <algorithm>
 
 #include "rkl_launch.h"
@@ -263,6 +265,22 @@ int sm_count()
     }
     return nsm;
 }
+// Whether the marching kernels of the face fluxes and of the advection (tiles of
+// 32 x 8 columns, `nzc` planes a thread, 3D) beat one thread per cell.  FP32:
+// idle lanes cost nothing while all warps are resident at once, and from eight
+// columns on the march's cheaper addressing outweighs them (rows of 4 cells, 368
+// x 41 of them: 0.8 of the speed; of 8, 805 x 20: 1.2).  FP64 runs at the FP64
+// rate either way, so idle lanes and uneven SMs are lost time and large grids of
+// full tiles gain 0-6% (flux: 256^3 3.59 -> 3.40 ms, but 64^3 62 against 68 us
+// and 40 x 208 x 123 0.23 against 0.35 ms).
+template <typename R>
+bool march_pays(const KGrid<R>& g, int nzc)
+{
+    if (g.plane >= ((int64_t)1 << 31) || g.n[1] > 8 * 65535) return false;
+    const int64_t warps = (int64_t)((g.n[0] + 31) / 32) * g.n[1] * ((g.n[2] + nzc - 1) / nzc);
+    if (sizeof(R) == 8) return g.n[0] % 32 == 0 && g.n[1] % 8 == 0 && warps >= 128 * (int64_t)sm_count();
+    return g.n[0] >= 8 || warps <= 16 * (int64_t)sm_count();
+}
 int generic_block(int64_t ncell)
 {
     int tpb = 256;
@@ -293,8 +311,8 @@ cudaError_t flux_impl(const void* grid, const void* phys, const void* T, const v
 {
     const KGrid<R>& g = *static_cast<const KGrid<R>*>(grid);
     const KPhys<R>& p = *static_cast<const KPhys<R>*>(phys);
-    if (NDIM == 3 && !p.limiter && g.plane < ((int64_t)1 << 31) && g.n[1] <= 8 * 65535) {
-        const int nzc = std::max(4, (g.n[2] + 65534) / 65535);
+    const int nzc = std::max(4, (g.n[2] + 65534) / 65535);
+    if (NDIM == 3 && !p.limiter && march_pays(g, nzc)) {
         const dim3 grid((g.n[0] + 31) / 32, (g.n[1] + 7) / 8, (g.n[2] + nzc - 1) / nzc);
         flux3_kernel<R, SPITZER, SAT><<<grid, 256, 0, st>>>(g, p, static_cast<const R*>(T), static_cast<const R*>(b),
                                                             static_cast<R*>(F[0]), static_cast<R*>(F[1]),
@@ -404,14 +422,13 @@ cudaError_t advect_impl(const LaunchCfg& c, const void* grid, const void* T, con
     const R* Tp = static_cast<const R*>(T);
     const R* up = static_cast<const R*>(u);
     R* op = static_cast<R*>(Tout);
+    // two planes per thread: more of them serialise the loads of a plane behind
+    // the last one's (7 planes: 24 us on 192 x 128 x 96)
+    const int nzc = std::max(2, (g.n[2] + 65534) / 65535);
     if (c.ndim == 1) advect_kernel<R, 1><<<blocks, tpb, 0, st>>>(g, Tp, up, op, (R)dt);
     else if (c.ndim == 2) advect_kernel<R, 2><<<blocks, tpb, 0, st>>>(g, Tp, up, op, (R)dt);
-    else if (g.plane < ((int64_t)1 << 31) && g.n[1] <= 8 * 65535) {
-        // two planes per thread: more of them serialise the loads of a plane
-        // behind the last one's (7 planes: 24 us on 192 x 128 x 96)
+    else if (march_pays(g, nzc)) {
         const dim3 xy((g.n[0] + 31) / 32, (g.n[1] + 7) / 8);
-        int nzc = 2;
-        nzc = std::max(nzc, (g.n[2] + 65534) / 65535);
         advect3_kernel<R><<<dim3(xy.x, xy.y, (g.n[2] + nzc - 1) / nzc), 256, 0, st>>>(g, Tp, up, op, (R)dt, nzc);
     } else advect_kernel<R, 3><<<blocks, tpb, 0, st>>>(g, Tp, up, op, (R)dt);
     return cudaGetLastError();
