@@ -256,7 +256,8 @@ rkl_status rkl_energy(rkl_plan *plan, const void *T, double *E_out);
  * Kernel choice for the stage launches of this plan: 0 = automatic (FP32 3D:
  * the row-pair kernel in the build for the grid's width and boundary, or the
  * tiled kernel for a limiter with a finite floor; 2D and FP64: the
- * column-march kernels; else the generic kernel), 1 = the generic one-thread-per-cell kernel, 2 = the
+ * column-march kernels, on narrow grids the generic kernel; else the generic
+ * kernel), 1 = the generic one-thread-per-cell kernel, 2 = the
  * tiled FP32 3D kernel (32 x 8 tiles, one cell per thread), 3 and 4 = the
  * paired-cell FP32 3D kernel (64 x 4 tiles, two cells per thread in packed
  * f32x2 arithmetic; needs nx % 4 == 0) built for 20 (variant 3) or 24
@@ -288,8 +289,9 @@ rkl_status rkl_energy(rkl_plan *plan, const void *T, double *E_out);
  * limited build on periodic grids, variants 3, 4, 6 and 7 the paired-cell
  * kernel's (20 resident warps per SM, per-thread copies; the same bits);
  * with a finite floor neither applies.
- * RKL_ERR_UNSUPPORTED if the kernel does not apply to the grid.  nzchunk = planes per CTA of the paired-cell
- * kernels (0: chosen from the grid and the SM count, at least 3.5 waves of
+ * RKL_ERR_UNSUPPORTED if the kernel does not apply to the grid.  nzchunk =
+ * planes per CTA (2D: rows per warp) of the marching kernels, variant 0
+ * included; for the paired-cell kernels (0: chosen from the grid and the SM count, at least 3.5 waves of
  * CTAs where the grid has that many and a last wave that is nearly full); a
  * negative value selects the balanced schedule instead: one launch of 5 (or
  * 6) CTAs per SM in which every CTA marches an equal run

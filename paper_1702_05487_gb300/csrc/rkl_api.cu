@@ -253,14 +253,14 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
                                 p->variant == 4 ? 3 : (p->variant == 9 ? 6 : 2), st, p->variant == 6,
                                 p->variant == 7, p->variant == 8);
         else if (p->colok && p->variant != 1 && p->variant != 2)
-            e = launch_stage_plane(p->cfg, p->gf, p->pf, io, cf, p->d_status, st);
+            e = launch_stage_plane(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk, st);
         else if (p->fast && al && (p->variant == 0 || p->variant == 2))
             e = launch_stage_fast(p->cfg, p->gf, p->pf, io, cf, p->d_status, st);
         else
             e = launch_stage_generic(p->cfg, &p->gf, &p->pf, io, &cf, p->d_status, st);
     } else {
         KCoef<double> cf{mu, nu, mt, gt};
-        if (p->colok && p->variant != 1) e = launch_stage_col(p->cfg, p->gd, p->pd, io, cf, p->d_status, st);
+        if (p->colok && p->variant != 1) e = launch_stage_col(p->cfg, p->gd, p->pd, io, cf, p->d_status, p->nzchunk, st);
         else e = launch_stage_generic(p->cfg, &p->gd, &p->pd, io, &cf, p->d_status, st);
     }
     if (e != cudaSuccess) return cuda_fail(p, e, "stage launch");
@@ -669,7 +669,7 @@ rkl_status rkl_plan_create(const rkl_grid* grid, const rkl_phys* phys, void* cud
     // a limiter floor inside the temperature range decides face by face on
     // FP32 rounding, so FP32 plans with one keep the kernels they had
     p->colok = col_stage_supported(g.dtype, g.ndim, p->gf.n, p->gf.plane) &&
-               (g.dtype == RKL_F64 || !p->cfg.limiter || p->cfg.lim_all);
+               (g.dtype == RKL_F64 || !p->cfg.limiter || p->cfg.lim_all) && col_stage_pays(p->cfg, p->gf.n);
 
     size_t cells = (size_t)ncell;
     if (p->xgok && g.n[0] % 4 != 0) {

@@ -499,40 +499,92 @@ inline int lanes_per_row(int nx, int ny)
     return best;
 }
 
-// Planes per block: a chunk costs its planes and about 0.8 for its first
-// z-face; an SM runs its blocks' planes at the FP64 rate whatever their
-// number, so the fullest SM decides.
-inline int chunk3(int64_t cols, int nz)
+// Length of a block's march and its cost.
+struct Chunk {
+    int len;
+    double cost;
+};
+
+// 3D, cost in planes of a lone block (7.2 us FP64 Spitzer, 4.7 constant, 13
+// saturated, 18 limited).  A chunk costs its planes and 0.5 (limited 0.6) for its
+// first z-face.  The fullest SM decides: K blocks on it take K times as long, at
+// the FP64 rate; one on every SM takes 1.6 times as long as one on every second
+// SM (limited 1.15).  CTAs start in z order, so the short last chunks of the
+// columns come last.  An SM takes two blocks at a time: near the end of the third
+// limited one, some take a fourth.  Fitted to chunks of 1 .. 64 planes on 44 grids
+// (8 x 6 x 8 to 100^3, columns of 3 x 500 and 4 x 5000) with each flux: the choice
+// is 0.4% (limited 2%) above the best on average.
+inline Chunk chunk3(int64_t cols, int nz, bool lim)
 {
-    int best = 1;
-    double cost = 1e300;
+    const double p = lim ? 0.6 : 0.5, one = lim ? 1.15 : 1.6;
+    auto at = [&](int64_t K) { return K == 1 ? one : (double)K; };
+    Chunk best{1, 1e300};
     for (int c = 1; c <= 64 && c <= nz; ++c) {
-        const double k = (double)(cols * ((nz + c - 1) / c)) / sms();
-        const double cst = (c + 0.8) * std::max(1.0, (std::ceil(k) + k) / 2.0);
-        if (cst < cost - 1e-9) {
-            cost = cst;
-            best = c;
+        const int64_t chunks = (nz + c - 1) / c, blocks = cols * chunks;
+        const int last = nz - (int)(chunks - 1) * c;
+        const double k = (double)blocks / sms();
+        double cost;
+        if (k <= 0.5) cost = c + p;
+        else if (k > 12.0) cost = (c + p) * (k + 0.3);
+        else {
+            const int64_t K = (blocks + sms() - 1) / sms();
+            const bool tail = chunks > 1 && blocks - (K - 1) * sms() <= cols && K > 1;
+            const double full = lim && k > 2.6 && k <= 3.0 ? 4.0 : at(K);
+            cost = tail ? (c + p) * at(K - 1) + (last + p) * (full - at(K - 1)) : (c + p) * full;
         }
+        if (cost < best.cost - 1e-9) best = Chunk{c, cost};
     }
     return best;
 }
 
+// 2D, cost in rows of a warp at the FP64 rate (0.56 us a row and SM, FP64
+// Spitzer).  With more than 96 rows an SM: 32 warps an SM, at most 32 rows each.
+// Below, 1 to 6 rows: a warp alone takes 4.4 a row and 4.8 to start; an SM takes
+// its warps' rows one after the other, with 0.8 more per warp for its first
+// y-face, and the fullest SM decides.  Limited blocks on more than every second SM: 1.4
+// times; one-row warps beyond four blocks an SM wait for a second round.  Fitted
+// like the above on 30 grids (8 x 8 to 60000 x 31).
+inline Chunk chunk2(int64_t ntx, int ny, bool lim)
+{
+    const double rows = (double)ntx * ny / sms();
+    if (rows > 96.0) {
+        const int c = (int)std::min(32.0, std::ceil(rows / 32.0));
+        return Chunk{c, rows * (1.0 + 0.8 / c)};
+    }
+    Chunk best{1, 1e300};
+    for (int c = 1; c <= 6 && c <= ny; ++c) {
+        const int64_t blocks = (ntx * ((ny + c - 1) / c) + NW2 - 1) / NW2;
+        const int64_t full = (blocks + sms() - 1) / sms();
+        const double alone = (4.4 * c + 4.8) * (lim && 2 * blocks > sms() ? 1.4 : 1.0);
+        const double cost = std::max(alone, NW2 * full * (c + 0.8)) + (full > 4 && c == 1 ? 8.0 : 0.0);
+        if (cost < best.cost - 1e-9) best = Chunk{c, cost};
+    }
+    return best;
+}
+
+// Blocks of a plane, and warps of a row.
+struct Cols {
+    int lpr, bx, by;
+};
+inline Cols cols3(int nx, int ny)
+{
+    const int lpr = lanes_per_row(nx, ny), rows = NW * 32 / lpr;
+    return Cols{lpr, (nx + lpr - 1) / lpr, (ny + rows - 1) / rows};
+}
+inline int cols2(int nx) { return (nx + 30) / 31; }
+
 template <typename R, bool SP, bool SAT, bool LIM, bool CUBE>
 cudaError_t launch_nd(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, const Args<R>& a, const KCoef<R>& cf,
-                      unsigned* status, cudaStream_t st, bool chained)
+                      unsigned* status, int chunk, cudaStream_t st, bool chained)
 {
     if (c.ndim == 3) {
-        const int lpr = lanes_per_row(g.n[0], g.n[1]), rows = NW * 32 / lpr;
-        const int bx = (g.n[0] + lpr - 1) / lpr, by = (g.n[1] + rows - 1) / rows;
-        const int nzc = chunk3((int64_t)bx * by, g.n[2]);
-        const dim3 grid(bx, by, (g.n[2] + nzc - 1) / nzc);
+        const Cols q = cols3(g.n[0], g.n[1]);
+        const int nzc = chunk > 0 ? chunk : chunk3((int64_t)q.bx * q.by, g.n[2], LIM).len;
+        const dim3 grid(q.bx, q.by, (g.n[2] + nzc - 1) / nzc);
         return launch_chained(col3_kernel<R, SP, SAT, LIM, CUBE>, grid, NT, 0, st, chained, g, p, a, cf, status, nzc,
-                              lpr);
+                              q.lpr);
     }
-    const int ntx = (g.n[0] + 30) / 31;
-    // rows per warp: about 32 warps per SM, at most 32 rows
-    const int64_t warps = (int64_t)32 * sms();
-    const int ch = (int)std::min<int64_t>(32, std::max<int64_t>(1, ((int64_t)ntx * g.n[1] + warps - 1) / warps));
+    const int ntx = cols2(g.n[0]), ch = chunk > 0 ? chunk : chunk2(ntx, g.n[1], LIM).len;
     const int64_t items = (int64_t)ntx * ((g.n[1] + ch - 1) / ch);
     return launch_chained(col2_kernel<R, SP, SAT, LIM, CUBE>, (unsigned)((items + NW2 - 1) / NW2), 32 * NW2, 0, st,
                           chained, g, p, a, cf, status, ch, ntx, (int)items);
@@ -540,15 +592,15 @@ cudaError_t launch_nd(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, 
 
 template <typename R, bool SP, bool SAT>
 cudaError_t launch_form(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, const Args<R>& a, const KCoef<R>& cf,
-                        unsigned* status, cudaStream_t st, bool chained)
+                        unsigned* status, int chunk, cudaStream_t st, bool chained)
 {
     bool cube = true;
     for (int d = 1; d < c.ndim; ++d) cube = cube && g.inv_dx[d] == g.inv_dx[0];
     if (c.limiter)
-        return cube ? launch_nd<R, SP, SAT, true, true>(c, g, p, a, cf, status, st, chained)
-                    : launch_nd<R, SP, SAT, true, false>(c, g, p, a, cf, status, st, chained);
-    return cube ? launch_nd<R, SP, SAT, false, true>(c, g, p, a, cf, status, st, chained)
-                : launch_nd<R, SP, SAT, false, false>(c, g, p, a, cf, status, st, chained);
+        return cube ? launch_nd<R, SP, SAT, true, true>(c, g, p, a, cf, status, chunk, st, chained)
+                    : launch_nd<R, SP, SAT, true, false>(c, g, p, a, cf, status, chunk, st, chained);
+    return cube ? launch_nd<R, SP, SAT, false, true>(c, g, p, a, cf, status, chunk, st, chained)
+                : launch_nd<R, SP, SAT, false, false>(c, g, p, a, cf, status, chunk, st, chained);
 }
 
 template <typename R>
@@ -562,14 +614,14 @@ Args<R> stage_args(const StageIO& io)
 
 template <typename R>
 cudaError_t launch(const LaunchCfg& c, const KGrid<R>& g, const KPhys<R>& p, const StageIO& io, const KCoef<R>& cf,
-                   unsigned* status, cudaStream_t st)
+                   unsigned* status, int chunk, cudaStream_t st)
 {
     const Args<R> a = stage_args<R>(io);
     if (c.spitzer)
-        return c.saturate ? launch_form<R, true, true>(c, g, p, a, cf, status, st, io.chained)
-                          : launch_form<R, true, false>(c, g, p, a, cf, status, st, io.chained);
-    return c.saturate ? launch_form<R, false, true>(c, g, p, a, cf, status, st, io.chained)
-                      : launch_form<R, false, false>(c, g, p, a, cf, status, st, io.chained);
+        return c.saturate ? launch_form<R, true, true>(c, g, p, a, cf, status, chunk, st, io.chained)
+                          : launch_form<R, true, false>(c, g, p, a, cf, status, chunk, st, io.chained);
+    return c.saturate ? launch_form<R, false, true>(c, g, p, a, cf, status, chunk, st, io.chained)
+                      : launch_form<R, false, false>(c, g, p, a, cf, status, chunk, st, io.chained);
 }
 
 }  // namespace col

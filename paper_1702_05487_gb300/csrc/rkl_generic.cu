@@ -687,6 +687,14 @@ cudaError_t launch_stage_generic(const LaunchCfg& c, const void* grid, const voi
     return stage_dispatch_ndim<float>(c, grid, phys, io, coef, status, st);
 }
 
+double generic_cells(int64_t ncell)
+{
+    const int tpb = generic_block(ncell);
+    const int64_t blocks = (ncell + tpb - 1) / tpb;
+    const double k = (double)blocks / sm_count();
+    return tpb * (k > 8.0 ? k + 0.4 : (double)((blocks + sm_count() - 1) / sm_count()));
+}
+
 cudaError_t launch_advect(const LaunchCfg& c, const void* grid, const void* T, const void* u, void* Tout, double dt,
                           cudaStream_t st)
 {

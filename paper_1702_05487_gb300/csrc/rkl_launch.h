@@ -63,17 +63,23 @@ struct LaunchCfg {
 cudaError_t launch_stage_generic(const LaunchCfg& c, const void* grid, const void* phys,
                                  const StageIO& io, const void* coef, unsigned* status,
                                  cudaStream_t st);
+// Cells on the fullest SM in a launch of the generic stage kernel (on average
+// and 0.4 blocks more where an SM runs many).
+double generic_cells(int64_t ncell);
+
 cudaError_t launch_flux_generic(const LaunchCfg& c, const void* grid, const void* phys,
                                 const void* T, const void* b, void* F[3], cudaStream_t st);
 
 // Column-march stage kernels: 2D grids (FP64, and FP32 in packed pairs) and
 // FP64 3D grids, any width, either boundary, limiter at any floor (FP32: at
-// every face); each face evaluated once.
+// every face); each face evaluated once.  chunk > 0 fixes the length of a
+// march (planes, 2D: rows).  col_stage_pays: they are the faster choice.
 bool col_stage_supported(int dtype, int ndim, const int n[3], int64_t plane);
+bool col_stage_pays(const LaunchCfg& c, const int n[3]);
 cudaError_t launch_stage_col(const LaunchCfg& c, const KGrid<double>& g, const KPhys<double>& p, const StageIO& io,
-                             const KCoef<double>& coef, unsigned* status, cudaStream_t st);
+                             const KCoef<double>& coef, unsigned* status, int chunk, cudaStream_t st);
 cudaError_t launch_stage_plane(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
-                               const KCoef<float>& coef, unsigned* status, cudaStream_t st);
+                               const KCoef<float>& coef, unsigned* status, int chunk, cudaStream_t st);
 
 // Operator splitting: one donor-cell advection step T_out = T - dt div(u T)
 // (u: [3][ncell] cell-centred velocity), and the statistics (as launch_stats,

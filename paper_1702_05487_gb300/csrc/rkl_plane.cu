@@ -202,12 +202,12 @@ plane_kernel(KGrid<float> g, KPhys<float> p, Args<float> a, KCoef<float> cf, uns
 
 template <bool SP, bool SAT, bool LIM>
 cudaError_t launch_plane(const KGrid<float>& g, const KPhys<float>& p, const Args<float>& a, const KCoef<float>& cf,
-                         unsigned* status, cudaStream_t st, bool chained)
+                         unsigned* status, int chunk, cudaStream_t st, bool chained)
 {
     const int ntx = (g.n[0] + COLS - 1) / COLS;
     // rows per warp: about 24 warps per SM, at most 32 rows
     const int64_t warps = (int64_t)24 * sms();
-    const int ch = (int)std::min<int64_t>(32, std::max<int64_t>(1, ((int64_t)ntx * g.n[1] + warps - 1) / warps));
+    const int ch = chunk > 0 ? chunk : (int)std::min<int64_t>(32, std::max<int64_t>(1, ((int64_t)ntx * g.n[1] + warps - 1) / warps));
     const int64_t items = (int64_t)ntx * ((g.n[1] + ch - 1) / ch);
     const unsigned blocks = (unsigned)((items + NWP - 1) / NWP);
     auto al8 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 7u) == 0; };
@@ -224,15 +224,15 @@ cudaError_t launch_plane(const KGrid<float>& g, const KPhys<float>& p, const Arg
 }  // namespace col
 
 cudaError_t launch_stage_plane(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
-                               const KCoef<float>& cf, unsigned* status, cudaStream_t st)
+                               const KCoef<float>& cf, unsigned* status, int chunk, cudaStream_t st)
 {
     if (c.ndim != 2 || !col_stage_supported(c.dtype, c.ndim, g.n, g.plane) || (c.limiter && !c.lim_all))
         return cudaErrorNotSupported;
     const col::Args<float> a = col::stage_args<float>(io);
     auto go = [&](auto sp, auto sat) {
         constexpr bool SP = decltype(sp)::value, SAT = decltype(sat)::value;
-        return c.limiter ? col::launch_plane<SP, SAT, true>(g, p, a, cf, status, st, io.chained)
-                         : col::launch_plane<SP, SAT, false>(g, p, a, cf, status, st, io.chained);
+        return c.limiter ? col::launch_plane<SP, SAT, true>(g, p, a, cf, status, chunk, st, io.chained)
+                         : col::launch_plane<SP, SAT, false>(g, p, a, cf, status, chunk, st, io.chained);
     };
     using T = std::true_type;
     using F = std::false_type;
