@@ -98,16 +98,33 @@ cudaError_t ensemble_launch_q(const x2::EnsProb* probs, const x2::EnsSeg* segs, 
 // 16 .. 64, the length that minimises (rounds of resident CTAs) x (planes +
 // halo cost), keeping the 3.5 waves (the paired-cell kernel's rule with this
 // kernel's tile and occupancy); down to one wave at 16 planes the same cost
-// without that floor.  Grids below one wave fill the chip with shorter
-// chunks: with k CTAs per SM (mean), a chunk costs its planes and 1.5 for its
-// prologue, and a plane costs one latency-bound step (2.2 units) until about
-// two CTAs share an SM, then the SM's throughput, between the mean k and the
-// fullest SM's ceil(k).  Constants fitted to a sweep of 1 .. 64 planes over
-// 32^3 .. 128^3 and two uneven boxes; the choice is within 4% of the best
-// length on each.  Stage time at 16 planes (the shortest chunk before) and
-// now: 32^3 14.2 -> 2.9 us, 64^3 11.6 -> 4.2, 96^3 14.5 -> 8.9, 128^3 15.7 ->
-// 14.4, 128^3 saturated 23.7 -> 19.1.
-int auto_nzchunk_q(const KGrid<float>& g, int tx, int ty)
+// without that floor.  Grids below one wave fill the chip with shorter chunks, a
+// chunk costing its planes and 1 for its prologue.  The fullest SM decides: of the
+// time of three CTAs (all that an SM holds) two take 0.84 and one alone 0.65 (the
+// classical flux on rows in 16-byte chunks: 0.75 and 0.5), a fourth starts the next round, and CTAs start in z order, so the short last
+// chunks come last.  Past six CTAs an SM the rounds blur: a third of the CTAs,
+// and a tenth more.  Fitted to 1 .. 64 planes on 34 boxes of 0.03 to 5 million
+// cells, classical, saturated and limited, in the periodic, DIR and PAD builds:
+// the choice is 1% above the best on average, 14%
+// at worst.  100 x 150 x 157 saturated, a stage: 34.9 us with the 10 planes of a rule
+// without rounds, now 28.8; 16 planes 31.9.  Stage time at 16 planes and now: 32^3 14.2 -> 2.9
+// us, 64^3 11.6 -> 4.2, 96^3 14.5 -> 8.9, 128^3 15.7 -> 14.4, 128^3 saturated 23.7
+// -> 19.1.
+double rounds_cost(int64_t cols, int nz, int nzc, int64_t sms, bool light)
+{
+    const double F[4] = {0.0, light ? 0.5 : 0.65, light ? 0.75 : 0.84, 1.0};
+    const int64_t chunks = (nz + nzc - 1) / nzc, ctas = cols * chunks;
+    const int last = nz - (int)(chunks - 1) * nzc;
+    const double k = (double)ctas / (double)sms;
+    if (k > 6.0) return (nzc + 1.0) * k / 3.0 * 1.1;
+    const int64_t K = (ctas + sms - 1) / sms, full = (K - 1) / kCtasPerSm;
+    const int r = (int)((K - 1) % kCtasPerSm) + 1;
+    if (chunks > 1 && ctas - sms * (K - 1) <= cols)       // the last to start are short ones
+        return (nzc + 1.0) * full + (last + 1.0) * F[r] + (r > 1 ? (nzc - last) * F[r - 1] : 0.0);
+    return (nzc + 1.0) * (full + F[r]);
+}
+
+int auto_nzchunk_q(const KGrid<float>& g, int tx, int ty, bool light)
 {
     const int64_t cols = (int64_t)((g.n[0] + tx - 1) / tx) * ((g.n[1] + ty - 1) / ty);
     const int64_t sms = sm_count(), slots = kCtasPerSm * sms;
@@ -116,15 +133,14 @@ int auto_nzchunk_q(const KGrid<float>& g, int tx, int ty)
     int best = 32;
     double cost = 1e300;
     for (int nzc = wave ? 16 : 1; nzc <= 64; ++nzc) {
-        const int64_t chunks = (g.n[2] + nzc - 1) / nzc;
         double cst;
         if (wave) {
+            const int64_t chunks = (g.n[2] + nzc - 1) / nzc;
             if (many && cols * chunks * 2 < 7 * slots) continue;
             const int64_t rounds = (cols * chunks + slots - 1) / slots;
             cst = (double)rounds * (std::min(nzc, g.n[2]) + 2.5);
         } else {
-            const double k = (double)(cols * chunks) / (double)sms;
-            cst = (std::min(nzc, g.n[2]) + 1.5) * std::max(2.2, (std::ceil(k) + 2.0 * k) / 3.0);
+            cst = rounds_cost(cols, g.n[2], std::min(nzc, g.n[2]), sms, light);
         }
         if (cst < cost - 1e-9) {
             cost = cst;
@@ -151,7 +167,8 @@ cudaError_t launch_stage_xq(const LaunchCfg& c, const KGrid<float>& g, const KPh
     const x2::FastArgs a = x2_args(io);
     // the limited build comes with 64-column tiles only
     if (c.limiter) txw = 64;
-    if (nzchunk <= 0) nzchunk = xq::auto_nzchunk_q(g, txw, txw == 64 ? xq::SmemQ<64>::TY : xq::SmemQ<32>::TY);
+    if (nzchunk <= 0) nzchunk = xq::auto_nzchunk_q(g, txw, txw == 64 ? xq::SmemQ<64>::TY : xq::SmemQ<32>::TY,
+                                                  !c.limiter && !c.saturate);
     if (c.limiter) return xq::launch_q_lim(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzchunk, st, io.chained);
     if (c.saturate)
         return xq::launch_q_sat(c.spitzer != 0, p.kperp == 0.f, txw, io.mode, g, p, a, coef, status, nzchunk, st, io.chained);
@@ -175,9 +192,11 @@ cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPh
 {
     if (!xg_stage_supported(c, g)) return cudaErrorNotSupported;
     const x2::FastArgs a = x2_args(io);
-    int nzc = nzchunk > 0 ? nzchunk : xq::auto_nzchunk_q(g, 64, xq::SmemQ<64>::TY);
+    const bool dir = g.bc == 1 && g.n[0] % 4 == 0;
+    int nzc = nzchunk > 0 ? nzchunk
+                          : xq::auto_nzchunk_q(g, 64, xq::SmemQ<64>::TY, dir && !c.limiter && !c.saturate);
     nzc = std::max(nzc, (g.n[2] + 65534) / 65535);      // the grid's z limit
-    if (g.bc == 1 && g.n[0] % 4 == 0)
+    if (dir)
         return (c.limiter ? xq::launch_q_dir_lim : xq::launch_q_dir)(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a,
                                                                      coef, status, nzc, st, io.chained);
     if (c.limiter) return xq::launch_q_gen_lim(c.spitzer != 0, c.saturate != 0, io.mode, g, p, a, coef, status, nzc, st, io.chained);
@@ -240,7 +259,7 @@ cudaError_t launch_stage_xp(const LaunchCfg& c, const KGrid<float>& g, const KPh
                             const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st)
 {
     if (!xg_stage_supported(c, g) || g.pitch % 4 != 0) return cudaErrorNotSupported;
-    int nzc = nzchunk > 0 ? nzchunk : xq::auto_nzchunk_q(g, 64, xq::SmemQ<64>::TY);
+    int nzc = nzchunk > 0 ? nzchunk : xq::auto_nzchunk_q(g, 64, xq::SmemQ<64>::TY, false);
     nzc = std::max(nzc, (g.n[2] + 65534) / 65535);      // the grid's z limit
     return (c.limiter ? xq::launch_q_pad_lim : xq::launch_q_pad)(c.spitzer != 0, c.saturate != 0, io.mode, g, p,
                                                                  x2_args(io), coef, status, nzc, st, io.chained);
