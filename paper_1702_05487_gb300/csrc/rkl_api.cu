@@ -55,6 +55,7 @@ struct rkl_plan {
     bool pairok = false;               // two-stage kernel applies to the grid
     bool xqok = false;                 // row-pair kernel applies to the grid
     bool xgok = false;                 // row-pair kernel for any width and boundary applies
+    bool xgpays = false;               // and is faster than the tiled one
     // FP32 3D widths that are not a multiple of four: super-steps run on
     // row-padded arrays (the plan's buffers and copies of T and b, allocated on
     // use), whose rows start 16-byte aligned
@@ -246,7 +247,7 @@ rkl_status launch_stage(rkl_plan* p, const StageIO& io, double mu, double nu, do
             const bool narrow = p->variant == 11 || (p->variant == 0 && narrow_tiles(p->gf.n[0]));
             e = launch_stage_xq(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk, st, narrow ? 32 : 64);
         }
-        else if (p->xgok && al && p->variant == 0)
+        else if (p->xgok && p->xgpays && al && p->variant == 0)
             e = launch_stage_xg(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk, st);
         else if (p->x2ok && al && (p->variant == 0 || (p->variant >= 3 && p->variant <= 9)))
             e = launch_stage_x2(p->cfg, p->gf, p->pf, io, cf, p->d_status, p->nzchunk,
@@ -666,6 +667,7 @@ rkl_status rkl_plan_create(const rkl_grid* grid, const rkl_phys* phys, void* cud
     p->pairok = g.dtype == RKL_F32 && pair_stage_supported(p->cfg, p->gf);
     p->xqok = g.dtype == RKL_F32 && xq_stage_supported(p->cfg, p->gf);
     p->xgok = g.dtype == RKL_F32 && xg_stage_supported(p->cfg, p->gf);
+    p->xgpays = p->xgok && (!p->fast || xg_stage_pays(p->cfg, p->gf));
     // a limiter floor inside the temperature range decides face by face on
     // FP32 rounding, so FP32 plans with one keep the kernels they had
     p->colok = col_stage_supported(g.dtype, g.ndim, p->gf.n, p->gf.plane) &&

@@ -135,6 +135,7 @@ cudaError_t launch_stage_xq(const LaunchCfg& c, const KGrid<float>& g, const KPh
 // every face, fewer than 2^31 cells, 16-byte aligned arrays; nzchunk <= 0
 // picks the chunk length.
 bool xg_stage_supported(const LaunchCfg& c, const KGrid<float>& g);
+bool xg_stage_pays(const LaunchCfg& c, const KGrid<float>& g);     // ... and is faster than the tiled kernel
 cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
                             const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st);
 

@@ -187,6 +187,19 @@ bool xg_stage_supported(const LaunchCfg& c, const KGrid<float>& g)
            g.n[1] <= 8 * 65535;
 }
 
+// GEN against the one-cell tiled kernel (32 x 8 tiles, an L1-served march that
+// skips what lies outside) on rows of a few cells, from one wave of CTAs on
+// (smaller grids need GEN's short chunks).  M of 500 x 500 rows with walls: 3
+// cells 304 against 226 us, 17 cells 0.88 and 31 cells 1.06 of its speed; periodic rows
+// of 1 cell 0.75, of 2 cells 1.26.
+bool xg_stage_pays(const LaunchCfg& c, const KGrid<float>& g)
+{
+    if (g.n[0] % 4 == 0) return true;                   // DIR
+    const int64_t at16 = (int64_t)((g.n[1] + 7) / 8) * ((g.n[2] + 15) / 16);
+    const int narrow = g.bc == 0 ? 1 : (c.limiter ? 12 : 20);
+    return g.n[0] > narrow || at16 < xq::kCtasPerSm * (int64_t)sm_count();
+}
+
 cudaError_t launch_stage_xg(const LaunchCfg& c, const KGrid<float>& g, const KPhys<float>& p, const StageIO& io,
                             const KCoef<float>& coef, unsigned* status, int nzchunk, cudaStream_t st)
 {

@@ -44,3 +44,33 @@ def test_narrow_grid_is_not_slower_than_generic(rk, dtype, shape, phys):  # noqa
         if auto < 1.12 * generic:
             return
     raise AssertionError((auto, generic))
+
+
+@pytest.mark.parametrize("shape,bc", [((500, 500, 3), "dirichlet"), ((500, 500, 1), "periodic"),
+                                      ((20, 3000, 9), "dirichlet")])
+def test_narrow_box_is_not_slower_than_tiled(rk, shape, bc):  # noqa: F811
+    """M of FP32 boxes a few cells wide against the one-cell tiled kernel
+    (variant 2); the row-pair kernel took 1.3 to 1.4 times as long."""
+    import torch
+    T = 1.0 + 0.2 * torch.rand(shape, device="cuda")
+    b = torch.rand((3,) + shape, device="cuda")
+    M = torch.empty_like(T)
+    plan = rk.Plan(shape, "f32", params=dict(SPITZ, bc=bc, bc_value=1.0, dx=(1.0 / max(shape),) * 3))
+
+    def best_ms(variant):
+        plan.set_variant(variant)
+        best = 1e300
+        for k in range(25):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            plan.apply_M(T, b, M)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1)) if k else best
+        return best
+
+    for _ in range(3):
+        tiled, auto = best_ms(2), best_ms(0)
+        if auto < 1.12 * tiled:
+            return
+    raise AssertionError((auto, tiled))
