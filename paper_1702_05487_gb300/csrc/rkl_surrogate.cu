@@ -32,6 +32,10 @@ constexpr int kLayers = 6;
 constexpr int kCout[kLayers] = {32, 32, 32, 32, 32, 16};
 constexpr int kCin[kLayers] = {16, 32, 32, 32, 32, 32};
 constexpr int kPartials = 1024;
+// What the host reads back sits in one block, so that a call makes one copy:
+// 2 kPartials FP64 partial sums, the bias gradients (32 a layer) and the status
+// word of the bounded waits.
+constexpr size_t kBackWords = 4 * kPartials + 32 * kLayers + 1;
 
 __global__ void axpy_kernel(const float* a, const float* b, float* out, int64_t n)
 {
@@ -116,10 +120,10 @@ struct rkl_surrogate {
     float* Mp = nullptr;
     int backend = 0;               // 0: warp-level mma.sync convolutions, 1: tcgen05
     unsigned* d_tcst = nullptr;    // status word of the tcgen05 kernels' bounded waits
-    unsigned* h_tcst = nullptr;    // as last read (pinned, behind h_part); kept until rkl_sur_check
+    unsigned* h_tcst = nullptr;    // as last read; kept until rkl_sur_check
     bool tc_unread = false;        // a layer's weight gradient was launched since
-    double* d_part = nullptr;
-    double* h_part = nullptr;      // pinned
+    double* d_part = nullptr;      // head of the read-back block
+    double* h_part = nullptr;      // the same block in pinned memory
     bool forward_done = false;
     double head_scale = 0.0;
     std::string err;
@@ -181,7 +185,6 @@ rkl_status backward_impl(rkl_surrogate* s, const float* target, double* loss)
     const int D = s->D, H = s->H, W = s->W;
     SUR_CK(s, conv::loss_and_adjoint(s->dT, target, D, H, W, (float)s->head_scale, s->inv_dx, s->d_part,
                                      kPartials, s->dG, s->stream));
-    SUR_CK(s, cudaMemcpyAsync(s->h_part, s->d_part, sizeof(double) * kPartials, cudaMemcpyDeviceToHost, s->stream));
     // head
     const void* dz = s->dG;
     SUR_CK(s, conv::conv_wgrad_tc(32, 16, dz, s->A[4], s->gw[5], s->gb[5], s->gpart, D, H, W, s->d_tcst, s->stream));
@@ -196,7 +199,7 @@ rkl_status backward_impl(rkl_surrogate* s, const float* target, double* loss)
             cur = 1 - cur;
         }
     }
-    SUR_CK(s, cudaMemcpyAsync(s->h_tcst, s->d_tcst, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
+    SUR_CK(s, cudaMemcpyAsync(s->h_part, s->d_part, 4 * kBackWords, cudaMemcpyDeviceToHost, s->stream));
     SUR_CK(s, cudaStreamSynchronize(s->stream));
     s->tc_unread = false;
     rkl_status st = grads_ok(s);
@@ -256,7 +259,7 @@ rkl_status rkl_sur_create(int D, int H, int W, const double* dx, void* cuda_stre
             if ((c = cudaMalloc(p, sizeof(float) * n)) != cudaSuccess) return bail(c, "params");
             if ((c = cudaMemsetAsync(*p, 0, sizeof(float) * n, s->stream)) != cudaSuccess) return bail(c, "params");
         }
-        float** fb[] = {&s->b[l], &s->gb[l], &s->mb[l], &s->vb[l]};
+        float** fb[] = {&s->b[l], &s->mb[l], &s->vb[l]};
         for (auto p : fb) {
             if ((c = cudaMalloc(p, sizeof(float) * nb)) != cudaSuccess) return bail(c, "bias");
             if ((c = cudaMemsetAsync(*p, 0, sizeof(float) * nb, s->stream)) != cudaSuccess) return bail(c, "bias");
@@ -277,14 +280,14 @@ rkl_status rkl_sur_create(int D, int H, int W, const double* dx, void* cuda_stre
     if ((c = cudaMalloc(&s->M0, (size_t)V * 4)) != cudaSuccess) return bail(c, "M0");
     if ((c = cudaMalloc(&s->Mp, (size_t)V * 4)) != cudaSuccess) return bail(c, "Mp");
     if ((c = cudaMalloc(&s->F3, (size_t)V * 12)) != cudaSuccess) return bail(c, "flux features");
-    if ((c = cudaMalloc(&s->d_part, sizeof(double) * 2 * kPartials)) != cudaSuccess) return bail(c, "partials");
+    if ((c = cudaMalloc(&s->d_part, 4 * kBackWords)) != cudaSuccess) return bail(c, "partials");
+    if ((c = cudaMemsetAsync(s->d_part, 0, 4 * kBackWords, s->stream)) != cudaSuccess) return bail(c, "partials");
+    for (int l = 0; l < kLayers; ++l) s->gb[l] = reinterpret_cast<float*>(s->d_part + 2 * kPartials) + 32 * l;
+    s->d_tcst = reinterpret_cast<unsigned*>(s->gb[0] + 32 * kLayers);
     if ((c = cudaMalloc(&s->gpart, sizeof(float) * conv::wgrad_workspace_floats())) != cudaSuccess)
         return bail(c, "gradient partials");
-    if ((c = cudaMalloc(&s->d_tcst, sizeof(unsigned))) != cudaSuccess) return bail(c, "status");
-    if ((c = cudaMemsetAsync(s->d_tcst, 0, sizeof(unsigned), s->stream)) != cudaSuccess) return bail(c, "status");
-    if ((c = cudaMallocHost(&s->h_part, sizeof(double) * (2 * kPartials + 1))) != cudaSuccess)
-        return bail(c, "partials");
-    s->h_tcst = reinterpret_cast<unsigned*>(s->h_part + 2 * kPartials);
+    if ((c = cudaMallocHost(&s->h_part, 4 * kBackWords)) != cudaSuccess) return bail(c, "partials");
+    s->h_tcst = reinterpret_cast<unsigned*>(s->h_part) + kBackWords - 1;
     *s->h_tcst = 0u;
     if ((c = cudaStreamSynchronize(s->stream)) != cudaSuccess) return bail(c, "sync");
     for (int l = 0; l < kLayers; ++l)
@@ -298,7 +301,7 @@ rkl_status rkl_sur_destroy(rkl_surrogate* s)
     if (!s) return RKL_ERR_INVALID_ARG;
     cudaStreamSynchronize(s->stream);
     for (int l = 0; l < kLayers; ++l) {
-        cudaFree(s->w[l]); cudaFree(s->b[l]); cudaFree(s->gw[l]); cudaFree(s->gb[l]);
+        cudaFree(s->w[l]); cudaFree(s->b[l]); cudaFree(s->gw[l]);
         cudaFree(s->mw[l]); cudaFree(s->vw[l]); cudaFree(s->mb[l]); cudaFree(s->vb[l]);
         cudaFree(s->wf[l]); cudaFree(s->wb[l]);
     }
@@ -309,7 +312,6 @@ rkl_status rkl_sur_destroy(rkl_surrogate* s)
     cudaFree(s->Yp); cudaFree(s->M0); cudaFree(s->Mp); cudaFree(s->F3);
     cudaFree(s->d_part);
     cudaFree(s->gpart);
-    cudaFree(s->d_tcst);
     if (s->h_part) cudaFreeHost(s->h_part);
     delete s;
     return RKL_OK;
@@ -341,11 +343,12 @@ rkl_status rkl_sur_get_grads(rkl_surrogate* s, int layer, float* gw_host, float*
 {
     if (!s || layer < 0 || layer >= kLayers || !gw_host || !gb_host) return RKL_ERR_INVALID_ARG;
     SUR_CK(s, cudaMemcpyAsync(gw_host, s->gw[layer], sizeof(float) * wcount(layer), cudaMemcpyDeviceToHost, s->stream));
-    SUR_CK(s, cudaMemcpyAsync(gb_host, s->gb[layer], sizeof(float) * kCout[layer], cudaMemcpyDeviceToHost, s->stream));
-    if (s->tc_unread)
-        SUR_CK(s, cudaMemcpyAsync(s->h_tcst, s->d_tcst, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
+    // the layer's bias gradient, those behind it and the status word
+    float* gb = reinterpret_cast<float*>(s->h_part + 2 * kPartials) + 32 * layer;
+    SUR_CK(s, cudaMemcpyAsync(gb, s->gb[layer], 4 * (32 * (kLayers - layer) + 1), cudaMemcpyDeviceToHost, s->stream));
     SUR_CK(s, cudaStreamSynchronize(s->stream));
     s->tc_unread = false;
+    std::memcpy(gb_host, gb, sizeof(float) * kCout[layer]);
     return grads_ok(s);
 }
 
