@@ -62,7 +62,7 @@ struct rkl_plan {
     bool padok = false;
     KGrid<float> gpad{};
     void* padT = nullptr;
-    void* padb = nullptr;
+    void* padb = nullptr;              // behind padT in one allocation
     bool colok = false;                // column-march kernel applies to the grid
     void* my0 = nullptr;
     double* d_partials = nullptr;
@@ -277,11 +277,13 @@ bool wants_padding(const rkl_plan* p, int s) { return p->padok && p->variant == 
 // only call single stages or short super-steps hold four grid arrays, not eight.
 void allocate_padding(rkl_plan* p)
 {
-    const size_t bytes = (size_t)p->gpad.ncell * p->esize;
-    if (cudaMalloc(&p->padT, bytes) == cudaSuccess && cudaMalloc(&p->padb, 3 * bytes) == cudaSuccess) return;
+    const size_t bytes = (size_t)p->gpad.ncell * p->esize;      // a multiple of 16
+    if (cudaMalloc(&p->padT, 4 * bytes) == cudaSuccess) {
+        p->padb = static_cast<char*>(p->padT) + bytes;
+        return;
+    }
     // no room: the stages read the caller's rows
     cudaGetLastError();
-    cudaFree(p->padT);
     p->padT = nullptr;
     p->padok = false;
 }
@@ -732,7 +734,6 @@ rkl_status rkl_plan_destroy(rkl_plan* p)
     for (int k = 0; k < 3; ++k) cudaFree(p->ybuf[k]);
     cudaFree(p->ybuf4);
     cudaFree(p->padT);
-    cudaFree(p->padb);
     cudaFree(p->my0);
     if (p->s_in) cudaStreamSynchronize(p->s_in);
     if (p->s_out) cudaStreamSynchronize(p->s_out);
