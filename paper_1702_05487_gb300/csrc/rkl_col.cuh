@@ -21,7 +21,8 @@
 // and integer checks of the result: about 95 FP64 operations per cell and
 // stage against about 305 in the generic kernel, which evaluates both faces
 // of every axis.  112 x 96 x 80 FP64 stage (Spitzer): generic 419 us, this
-// kernel 176 us; 100 x 100 Dirichlet 8.2 -> 3.1 us.
+// kernel 176 us; 100 x 100 Dirichlet 8.2 -> 3.1 us.  Narrow grids stay with the
+// generic kernel (col_stage_pays).
 #pragma once
 
 #include <algorithm>

@@ -26,7 +26,8 @@
 // threads issue MMAs (one per dx, each into its own TMEM block, so that one
 // thread's waits and commits hide behind the others' MMAs), eight warps copy
 // (cp.async, three steps in flight, proxy fence once landed), one warp adds
-// up dz for the bias.  Every wait is bounded and reports ST_TIMEOUT.
+// up dz for the bias.  Every wait is bounded and reports ST_TIMEOUT, which the
+// calls that hand out or use the gradients turn into RKL_ERR_TIMEOUT.
 //
 // 32 -> 32 channels: 128^3 121 us with the slices' sum (the warp-level
 // mma.sync kernel before it: about 360), 96^3 64 us (about 180).  The MMAs alone

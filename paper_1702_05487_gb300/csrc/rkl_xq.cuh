@@ -40,11 +40,13 @@
 // aligned in global memory only if nx % 4 == 0; each lane's wrapped or clamped
 // column and row offsets are fixed per tile, Dirichlet ghosts of T are stored,
 // not copied.  33 copies a thread and plane instead of 9 throttle the memory
-// pipe (MIO stalls 1.6 cycles an issue against 0.2), so the single-stage entry
-// points take GEN, while super-steps take DIR or PAD.  201 x 150 x 99 stage:
-// one-cell tiled kernel 138 us, GEN 38, PAD 31 (and 20 us a super-step for the
-// copies).  Dirichlet 192 x 128 x 96, constant kappa: paired-cell 29 us, GEN
-// 22, DIR 16.
+// pipe (MIO stalls 1.6 cycles an issue against 0.2), so Dirichlet widths that are
+// a multiple of four always take DIR, and other widths take PAD in super-steps of
+// four stages or more (GEN in shorter ones and in single stages, unless the rows
+// are so short that the one-cell tiled kernel is faster, xg_stage_pays).  201 x
+// 150 x 99 stage: one-cell tiled kernel 138 us (saturated 147, limited 161), GEN
+// 38, PAD 31 (42, 43) and 20 us a super-step for the copies.  Dirichlet 192 x 128
+// x 96: paired-cell 27 us (saturated 32, limited 33), GEN 22, DIR 17 (24, 26).
 #pragma once
 
 #include <algorithm>
